@@ -87,13 +87,17 @@ typedef enum {
 } coffee_form;
 
 /* Arithmetic of the contraction A_e = sum_k G_e[k] T[k] (per-cell factors G, reference
- * tensors T), accumulated in FP32 on the tensor cores, float output; FP64: CUDA-core FP64,
- * double output. Each operand is held as a sum of parts of the operand type, each part the
+ * tensors T), accumulated in FP32 on the tensor cores, float output; FP64: double output, to
+ * double rounding (below). Each operand is held as a sum of parts of the operand type, each part the
  * round-to-nearest of what the previous ones left:
  *   TF32:   T and G one tf32 part each, one product;
  *   TF32X3: T and G two tf32 parts each, the three products hi*hi + hi*lo + lo*hi;
  *   BF16:   T two bf16 parts, G one, two products;
  *   BF16X3: T and G three bf16 parts each, the six products of order <= 2.
+ * FP64 runs on the CUDA cores, except where exact digit products on the tensor cores are faster
+ * (triangles and tetrahedra: MASS on 10 or more nodes, HELMHOLTZ and ADVDIFF on 4 or more): every
+ * operand as a fixed-point number of 61 or more bits, products and sums in integers, one rounding.
+ * COFFEE_FLAG_CUDA_CORES keeps FP64 on the plain one-thread-per-cell kernel.
  * Parity bounds (max |A - A_exact| / max |A_exact| per cell): 1e-5 for TF32X3 and BF16X3,
  * 1e-2 for TF32 and BF16. */
 typedef enum {
@@ -181,7 +185,7 @@ int coffee_tabulate(int cell, int degree, int quad_degree, int* nq, int* ndof,
  * Pass T = NULL to query *K and *N. */
 int coffee_reference_tensor(int form, int degree, int cell, int* K, int* N, double* T);
 
-/* FP64 local assembly (plain one-thread-per-cell kernel), all pointers on the device:
+/* FP64 local assembly (COFFEE_FP64 of coffee_assemble_ex), all pointers on the device:
  *   coords    [nverts][d] double
  *   cell2vert [ncells][d+1] int32 (prisms: [ncells][6])
  *   coef      ADVDIFF: [ncoefnodes][1+d] double, row = (eps, b_0, .., b_{d-1})
@@ -259,12 +263,12 @@ int coffee_round_coef(const double* coef, int64_t n, float* out, coffee_stream_t
 int coffee_supported(int form, int degree, int cell, int precision);
 
 /* The kernel family coffee_assemble_ex runs for local assembly with these arguments and flags:
- * 0 the FP64 kernel, 1 the tensor cores (tcgen05), 2 the FP32 CUDA-core kernel for small
+ * 0 the FP64 kernels, 1 the tensor cores (tcgen05), 2 the FP32 CUDA-core kernel for small
  * element matrices (COFFEE_FLAG_TENSOR_CORES / COFFEE_FLAG_CUDA_CORES); COFFEE_ERR_UNSUPPORTED
  * where coffee_supported is 0. Host-only. */
 int coffee_assemble_path(int form, int degree, int cell, int precision, unsigned flags);
 
-/* Local assembly (section 2, Listings 1-2) with a chosen precision. FP64 runs the plain FP64 kernel; the
+/* Local assembly (section 2, Listings 1-2) with a chosen precision. FP64 runs the FP64 kernels; the
  * other precisions run the tcgen05 tensor-core contraction with geometry fused into
  * its producer warps (FP32 geometry, FP64 for ill-conditioned cells).
  * Returns COFFEE_ERR_UNSUPPORTED for combinations without a kernel. */

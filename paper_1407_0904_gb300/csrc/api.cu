@@ -133,11 +133,18 @@ struct TcEntry {
   TcTable meta{};
 };
 
+struct DigitEntry {
+  uint8_t* image = nullptr;
+  int32_t* y20 = nullptr;
+  int32_t tk20[2] = {0, 0};
+};
+
 struct DeviceCache {
   unsigned* err = nullptr;
   int num_sms = 0;
   std::map<std::tuple<int, int, int>, double*> fp64;    // (form, degree, cell)
   std::map<std::tuple<int, int, int, int>, TcEntry> tc;  // + precision
+  std::map<std::tuple<int, int, int>, DigitEntry> digits;  // FP64 on the tensor cores
 };
 
 std::mutex g_mu;
@@ -192,6 +199,34 @@ int fp64_table(DeviceCache& c, int form, int degree, int cell, const double** T)
   }
   c.fp64[key] = d;
   *T = d;
+  return COFFEE_OK;
+}
+
+int digit_table(DeviceCache& c, int form, int degree, int cell, Fp64Params& p) {
+  auto key = std::make_tuple(form, degree, cell);
+  auto it = c.digits.find(key);
+  if (it == c.digits.end()) {
+    std::vector<uint8_t> img;
+    std::vector<int32_t> y20;
+    DigitEntry ent;
+    build_fp64_image(form, degree, cell, img, y20, ent.tk20);
+    const size_t at = (img.size() + 15) & ~size_t(15), bytes = at + y20.size() * sizeof(int32_t);
+    img.resize(bytes);
+    std::memcpy(img.data() + at, y20.data(), y20.size() * sizeof(int32_t));
+    cudaError_t e = cudaMalloc(&ent.image, bytes);
+    if (e != cudaSuccess) return cuda_fail(e, "cudaMalloc(digit table)");
+    e = cudaMemcpy(ent.image, img.data(), bytes, cudaMemcpyHostToDevice);
+    if (e != cudaSuccess) {
+      cudaFree(ent.image);
+      return cuda_fail(e, "cudaMemcpy(digit table)");
+    }
+    ent.y20 = reinterpret_cast<int32_t*>(ent.image + at);
+    it = c.digits.emplace(key, ent).first;
+  }
+  p.digits = it->second.image;
+  p.yexp20 = it->second.y20;
+  p.tk20[0] = it->second.tk20[0];
+  p.tk20[1] = it->second.tk20[1];
   return COFFEE_OK;
 }
 
@@ -365,6 +400,13 @@ int assemble_impl(const coffee_assemble_args* a, const uint32_t* map, int64_t nn
     p.validate = validate ? 1 : 0;
     p.map = map;
     p.nnz = nnz;
+    // the digit contraction on the tensor cores where it is faster, unless the CUDA cores are asked for
+    if (!(a->flags & COFFEE_FLAG_CUDA_CORES) && fp64_tc_use(a->form, a->degree, a->cell)) {
+      if ((rc = digit_table(*c, a->form, a->degree, a->cell, p)) != COFFEE_OK) return rc;
+      cudaError_t e = (cudaError_t)launch_fp64_tc(a->form, a->cell, p, c->num_sms, stream);
+      if (e != cudaSuccess) return cuda_fail(e, "launch(assemble_fp64_tc)");
+      return COFFEE_OK;
+    }
     cudaError_t e = (cudaError_t)launch_fp64(a->form, a->cell, p, stream);
     if (e != cudaSuccess) return cuda_fail(e, "launch(assemble_fp64)");
     return COFFEE_OK;

@@ -74,9 +74,17 @@ struct Fp64Params {
   int validate;
   const uint32_t* map;  // global assembly: CSR position of every entry (blocked, csr_map_index), else NULL
   int64_t nnz;          // length of the CSR value array (out) when map is set
+  const uint8_t* digits;  // tensor-core kernel: digit image of T, the entries' exponents and the scales
+  const int32_t* yexp20;  // of the two kinds of factors (exponents << 20)
+  int32_t tk20[2];
 };
 // returns cudaError_t as int
 int launch_fp64(int form, int cell, const Fp64Params& p, void* stream);
+// FP64 on the tensor cores by exact digit products (k_fp64_tc.cu)
+int fp64_tc_use(int form, int degree, int cell);
+void build_fp64_image(int form, int degree, int cell, std::vector<uint8_t>& img, std::vector<int32_t>& y20,
+                      int32_t (&tk20)[2]);
+int launch_fp64_tc(int form, int cell, const Fp64Params& p, int num_sms, void* stream);
 
 // ---- FP64 prism kernel (k_prism.cu) ----
 struct PrismParams {

@@ -14,55 +14,10 @@
 //      tensors T (the quadrature loop pre-summed on the host).
 #include <cuda_runtime.h>
 #include "coffee_internal.h"
+#include "fp64_common.cuh"
 
 namespace coffee {
 namespace {
-
-template <int D>
-struct Geo {
-  double adj[D][D];  // adjugate: K = adj / det
-  double det;
-};
-
-template <int D>
-__device__ __forceinline__ void geometry64(const double (&X)[D + 1][D], Geo<D>& g) {
-  double J[D][D];
-#pragma unroll
-  for (int r = 0; r < D; ++r)
-#pragma unroll
-    for (int c = 0; c < D; ++c) J[r][c] = X[c + 1][r] - X[0][r];
-  if constexpr (D == 2) {
-    g.det = J[0][0] * J[1][1] - J[0][1] * J[1][0];
-    g.adj[0][0] = J[1][1];
-    g.adj[0][1] = -J[0][1];
-    g.adj[1][0] = -J[1][0];
-    g.adj[1][1] = J[0][0];
-  } else {
-    // cofactors C[r][c]; adj[a][r] = C[r][a]
-    double C00 = J[1][1] * J[2][2] - J[1][2] * J[2][1];
-    double C01 = J[1][2] * J[2][0] - J[1][0] * J[2][2];
-    double C02 = J[1][0] * J[2][1] - J[1][1] * J[2][0];
-    double C10 = J[0][2] * J[2][1] - J[0][1] * J[2][2];
-    double C11 = J[0][0] * J[2][2] - J[0][2] * J[2][0];
-    double C12 = J[0][1] * J[2][0] - J[0][0] * J[2][1];
-    double C20 = J[0][1] * J[1][2] - J[0][2] * J[1][1];
-    double C21 = J[0][2] * J[1][0] - J[0][0] * J[1][2];
-    double C22 = J[0][0] * J[1][1] - J[0][1] * J[1][0];
-    g.det = J[0][0] * C00 + J[0][1] * C01 + J[0][2] * C02;
-    g.adj[0][0] = C00; g.adj[0][1] = C10; g.adj[0][2] = C20;
-    g.adj[1][0] = C01; g.adj[1][1] = C11; g.adj[1][2] = C21;
-    g.adj[2][0] = C02; g.adj[2][1] = C12; g.adj[2][2] = C22;
-  }
-}
-
-template <int FORM, int D>
-struct FormK {
-  static constexpr int P = D * (D + 1) / 2;
-  static constexpr int value = FORM == FORM_MASS ? 1
-                               : FORM == FORM_HELMHOLTZ ? 1 + P
-                               : FORM == FORM_ADVDIFF ? (D + 1) * P + (D + 1) * D
-                                                      : 1;
-};
 
 // CSR: global assembly -- every entry is added into the CSR value array p.out at the
 // position p.map[cell][entry] instead of being stored.
