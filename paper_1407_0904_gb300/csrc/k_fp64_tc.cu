@@ -22,24 +22,21 @@
 // over cells relative to max|A_e|: Helmholtz P3 tetrahedra 2.2e-17 (plain kernel 2.5e-17), advection-
 // diffusion P2 4.4e-17 (6.3e-17), and no larger than the plain kernel's for any form, degree and cell.
 //
-// Digits are laid out so that an order is ONE contiguous K-run on both sides: the cell's digits
-// G_0, G_1, .. ascend, the table's descend, T_(ND-1), .., T_0, so order d pairs the first d+1 digit
-// blocks of the cell with the last d+1 of the table. Operands are K-major without swizzle, 16 bytes
-// (8 factors of one digit) per row and chunk, rows contiguous.
+// Operands are K-major without swizzle: 16-byte rows (8 factors of one digit) contiguous in chunks; T by
+// 128-entry slice, digit and chunk, the cells by chunk, digit and cell (see the MMA warp for why).
 //
 // One persistent CTA per SM holds two independent pipelines (halves), which keeps one busy while the
 // other waits: in each, three producer warps gather, form the factors in FP64 and store digits, a tile of
-// 32 cells each; one warp issues the MMAs (M = 128 entries, N = 32 cells) two units of two orders at a
-// time; eight epilogue warps (32 entries x 16 cells each) combine the orders in registers and write rows
-// of 32 doubles, 256 bytes. T's digits stay in shared memory where they fit; otherwise the CTAs split
+// 32 cells each; one warp issues the MMAs (M = 128 entries, N = 32 cells times digits); eight epilogue warps
+// (32 entries x 16 cells each) combine the orders in registers and write rows of 32 doubles, 256 bytes. T's digits stay in shared memory where they fit; otherwise the CTAs split
 // into groups by 128-entry slices, each with its slices resident, and form the factors once per group.
 // What bounds it now is the integer work of the epilogue, about 26 instructions an entry (half of them
 // moved to the multiplier pipe, see mad_lo), and the latencies between its phases. 196,608 tetrahedra,
-// this kernel / plain: Helmholtz P2 55 / 300 us, P3 167 / 1131 us (0.56 of the copy bandwidth), P4 416 /
-// 3310 us; advection-diffusion P2 168 / 1450 us, P4 1.43 / 16.9 ms. Steps on the way (Helmholtz P3): one
+// this kernel / plain: Helmholtz P2 57 / 300 us, P3 158 / 1131 us (0.6 of the copy bandwidth), P4 417 /
+// 3310 us; advection-diffusion P2 123 / 1450 us, P4 1.10 / 16.9 ms. Steps on the way (Helmholtz P3): one
 // pipeline with 21 warps 479 us; 16 warps of 128 registers 324; multiplications for shifts 311; two
-// pipelines 242; descriptors in uniform registers (the issuing thread took 110 cycles an MMA) and 16 cells
-// per epilogue warp, four epilogue warps a scheduler, 169.
+// pipelines 242; 16 cells per epilogue warp, four epilogue warps a scheduler, 169; one wide MMA per digit of T
+// instead of one per order and K step 158 (advection-diffusion P2 168 -> 123).
 // Cells whose factors are not finite or outside 2^+-900 are evaluated entry by entry in FP64.
 #include <cuda_runtime.h>
 #include <cuda_fp16.h>
@@ -50,6 +47,7 @@
 #include "coffee_internal.h"
 #include "tc_common.cuh"
 #include "fp64_common.cuh"
+#include "digits.cuh"
 
 namespace coffee {
 namespace {
@@ -64,15 +62,14 @@ constexpr int F_PROD = 3;              // producer warps of a half, a tile each 
 constexpr int F_PWARP0 = F_HALVES * F_EPI, F_MWARP0 = F_PWARP0 + F_HALVES * F_PROD;
 constexpr int F_WARPS = F_MWARP0 + F_HALVES;  // 24: six per scheduler, 80 registers a thread
 constexpr int F_THREADS = F_WARPS * 32;
-constexpr int F_UNITS = 4;             // accumulator units of a half: two orders (columns 0-31 and 32-63) each
+constexpr int F_COLS = 256;            // accumulator columns of a half: order d at columns 32 d
 constexpr int F_XRING = 8;             // tiles whose cell exponents are kept (operand stages + 2 at least)
 constexpr int F_STAGES = 4;            // operand stages of a half at most
 constexpr int CELL_SKIP = INT32_MIN, CELL_PLAIN = INT32_MIN + 1;
 constexpr uint32_t MAGIC = 0x4B400000u;  // 1.5 * 2^23 as a float
 
 struct alignas(8) FBars {
-  uint64_t full[F_HALVES][F_STAGES], empty[F_HALVES][F_STAGES], tfull[F_HALVES][F_UNITS], tempty[F_HALVES][F_UNITS],
-      done[F_HALVES];
+  uint64_t full[F_HALVES][F_STAGES], empty[F_HALVES][F_STAGES], tfull[F_HALVES], tempty[F_HALVES], done[F_HALVES];
   uint32_t tmem_base;
 };
 
@@ -83,123 +80,15 @@ struct Digits {
   static constexpr int ND = FORM == FORM_ADVDIFF ? 8 : 7;  // digits
   static constexpr int FB = FORM == FORM_ADVDIFF ? 62 : 61;  // fraction bits of the fixed-point operands
   static constexpr int KC = (K + 1 + 7) / 8;               // 8-factor chunks per digit, one slot for the constant
-  static constexpr int BCH = ND * KC + ((ND * KC) & 1);    // chunks of a cell row (MMAs take two)
   static constexpr int ACH = ND * KC + 1;                  // chunks of a table row, the last one zero
   static constexpr int SLICE = ACH * BM * 16;              // bytes of one 128-entry slice of the table
-  static constexpr int STAGE = BCH * FN * 16;
+  static constexpr int STAGE = ND * KC * FN * 16;
   COFFEE_HD static constexpr uint64_t bias() {
     uint64_t s = 0;
     for (int p = 0; p < ND; ++p) s += 1ull << (B - 1 + B * p);
     return s;
   }
 };
-
-__device__ __forceinline__ uint64_t f_desc(uint32_t saddr, uint32_t lbo) {
-  return (uint64_t)((saddr >> 4) & 0x3FFFu) | (uint64_t)((lbo >> 4) & 0x3FFFu) << 16 | (uint64_t)(128u >> 4) << 32 |
-         1ull << 46;
-}
-
-// tcgen05.mma (f16) and commit by one lane of a converged warp
-__device__ __forceinline__ void f_mma(uint32_t lead, uint32_t d, uint64_t ad, uint64_t bd, uint32_t idesc, uint32_t acc) {
-  asm volatile(
-      "{\n\t.reg .pred p, q;\n\tsetp.ne.b32 p, %4, 0;\n\tsetp.ne.b32 q, %5, 0;\n\t"
-      "@q tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(d),
-      "l"(ad), "l"(bd), "r"(idesc), "r"(acc), "r"(lead)
-      : "memory");
-}
-__device__ __forceinline__ void f_commit(uint32_t lead, uint32_t bar) {
-  asm volatile(
-      "{\n\t.reg .pred q;\n\tsetp.ne.b32 q, %1, 0;\n\t"
-      "@q tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n\t}" ::"r"(bar), "r"(lead)
-      : "memory");
-}
-
-// Fixed point of x scaled by 2^(FB - X), FB = 61 (b = 9) or 62 (b = 8): X = biased exponent bound of the
-// cell's factors (x < 2^(X-1022)), sh = X - (x's biased exponent) >= 0, plus the digits' bias.
-template <uint64_t BIAS, int FB>
-__device__ __forceinline__ uint64_t fixed_point(double x, int e20, int t20) {
-  const uint32_t h = (uint32_t)__double2hiint(x), l = (uint32_t)__double2loint(x);
-  const uint32_t ef = h & 0x7FF00000u;
-  const uint32_t sh = min(((uint32_t)(e20 - t20) - ef) >> 20, 63u);
-  uint64_t m = ((uint64_t)((h & 0xFFFFFu) | 0x100000u) << 32) | l;
-  m = ef == 0u ? 0ull : (m << (FB - 53)) >> sh;  // subnormals count as zero (the largest factor is above 2^-900)
-  return ((int)h < 0 ? 0ull - m : m) + BIAS;
-}
-
-// Eight factors' digits p = 0 (leading) .. ND-1 into chunk c of every digit block of a cell row.
-template <int B, int ND, int KC>
-__device__ __forceinline__ void store_digits(uint8_t* row, int c, const uint64_t (&U)[8], bool constant) {
-  constexpr uint32_t mask = (1u << B) - 1u;
-  // 0x6400 + u is the half 1024 + u, so one packed subtraction leaves the balanced digits
-  const __half2 off = __halves2half2(__ushort_as_half(0x6400 + (1 << (B - 1))), __ushort_as_half(0x6400 + (1 << (B - 1))));
-#pragma unroll
-  for (int p = 0; p < ND; ++p) {
-    const int sh = B * (ND - 1 - p);
-    uint32_t w[4];
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const uint32_t a = (uint32_t)(U[2 * j] >> sh), b = (uint32_t)(U[2 * j + 1] >> sh);
-      // the leading digit takes every bit left (b = 9: up to 2^9 at |g| = 2^62)
-      const uint32_t u = (p ? a & mask : a) | ((p ? b & mask : b) << 16) | 0x64006400u;
-      __half2 v = __hsub2(*reinterpret_cast<const __half2*>(&u), off);
-      w[j] = *reinterpret_cast<uint32_t*>(&v);
-    }
-    // the constant's factor, 4096, in the last slot of the leading digit block
-    if (constant) w[3] = (w[3] & 0xFFFFu) | (p == 0 ? 0x6C000000u : 0u);
-    *reinterpret_cast<uint4*>(row + (size_t)(p * KC + c) * FN * 16) = make_uint4(w[0], w[1], w[2], w[3]);
-  }
-}
-
-// Integer multiply-adds. The compiler would turn multiplications by known powers of two into shifts, which
-// share the ALU pipe (half a warp instruction per cycle) with everything else here; multiplications have
-// a pipe of their own, so the powers are kept in registers whose values it does not see.
-__device__ __forceinline__ uint32_t opaque(uint32_t x) {
-  uint32_t r;
-  asm("mov.u32 %0, %1;" : "=r"(r) : "r"(x));
-  return r;
-}
-__device__ __forceinline__ uint32_t mad_lo(uint32_t a, uint32_t b, uint32_t c) {
-  uint32_t r;
-  asm("mad.lo.u32 %0, %1, %2, %3;" : "=r"(r) : "r"(a), "r"(b), "r"(c));
-  return r;
-}
-__device__ __forceinline__ uint32_t mad_hi(uint32_t a, uint32_t b, uint32_t c) {
-  uint32_t r;
-  asm("mad.hi.u32 %0, %1, %2, %3;" : "=r"(r) : "r"(a), "r"(b), "r"(c));
-  return r;
-}
-__device__ __forceinline__ uint64_t mad_wide(uint32_t a, uint32_t b, uint64_t c) {
-  uint64_t r;
-  asm("mad.wide.u32 %0, %1, %2, %3;" : "=l"(r) : "r"(a), "r"(b), "l"(c));
-  return r;
-}
-
-// The double S 2^E, rounded to nearest (ties away), by integer instructions: S = hi:lo a two's complement
-// number below 2^62 with a high word other than 0 or -1 (bit < 0 otherwise, the result void),
-// e20 = (E + 1054) << 20; p22 = 2^22, p20 = 2^20. |S| is shifted to 2^62 <= m < 2^63, half a unit of the
-// last place (2^9) added on the way, and m >> 10 is the significand with its leading one, which counts as
-// one in the exponent field.
-__device__ __forceinline__ double from_fixed(uint32_t hi, uint32_t lo, uint32_t e20, uint32_t p22, uint32_t p20,
-                                             int& bit) {
-  const uint32_t s = (uint32_t)((int)hi >> 31);
-  asm("bfind.s32 %0, %1;" : "=r"(bit) : "r"(hi));  // the leading bit of |S| is 32 + bit
-  uint32_t P;
-  asm("shr.u32 %0, %1, %2;" : "=r"(P) : "r"(0x40000000u), "r"(bit));  // (0 for a bit of -1)
-  const uint64_t m = mad_wide(lo ^ s, P, 0x200ull);
-  const uint32_t mh = mad_lo(hi ^ s, P, (uint32_t)(m >> 32));
-  const uint32_t qh = mad_hi(mh, p22, mad_lo((uint32_t)bit, p20, e20));
-  return __hiloint2double((int)(qh | (s & 0x80000000u)), (int)__funnelshift_r((uint32_t)m, mh, 10));
-}
-// The same for any S below 2^62.
-__device__ __forceinline__ double from_fixed_any(uint32_t hi, uint32_t lo, uint32_t e20) {
-  int bit;
-  const uint32_t s = (uint32_t)((int)hi >> 31);
-  if ((hi ^ s) != 0u) return from_fixed(hi, lo, e20, 1u << 22, 1u << 20, bit);
-  const uint32_t l = lo ^ s;  // |S|, or |S| - 1
-  if (l < 4u) return 0.0;      // rounding of the digits
-  // 32 places up: |S| < 2^32 becomes 2^30 times itself, so that the high word stays below 2^30
-  return from_fixed(((l >> 2) ^ s), ((l << 30) ^ s), e20 - (30u << 20), 1u << 22, 1u << 20, bit);
-}
 
 template <int FORM, int D>
 __device__ __noinline__ double plain_entry(const Fp64Params& p, int64_t e, int o) {
@@ -219,9 +108,9 @@ __global__ void __launch_bounds__(F_THREADS, 1) k_assemble_fp64_tc(const Fp64Par
   using DG = Digits<FORM, D>;
   constexpr int K = DG::K, KC = DG::KC, ND = DG::ND, B = DG::B;
   extern __shared__ __align__(1024) uint8_t smem_raw[];
-  uint8_t* sA = smem_raw;
-  uint8_t* sB = sA + slices * DG::SLICE;
-  int* sX = reinterpret_cast<int*>(sB + F_HALVES * nst * DG::STAGE);
+  uint8_t* sB = smem_raw;
+  uint8_t* sA = sB + F_HALVES * nst * DG::STAGE;
+  int* sX = reinterpret_cast<int*>(sA + slices * DG::SLICE);
   FBars* bars = reinterpret_cast<FBars*>(sX + F_HALVES * F_XRING * FN);
 
   const int warp = __shfl_sync(0xffffffffu, (int)threadIdx.x >> 5, 0);  // known to be uniform
@@ -241,10 +130,8 @@ __global__ void __launch_bounds__(F_THREADS, 1) k_assemble_fp64_tc(const Fp64Par
         mbar_init(smem_u32(&bars->full[h][s]), FN);
         mbar_init(smem_u32(&bars->empty[h][s]), 1);
       }
-      for (int r = 0; r < F_UNITS; ++r) {
-        mbar_init(smem_u32(&bars->tfull[h][r]), 1);
-        mbar_init(smem_u32(&bars->tempty[h][r]), F_EPI);
-      }
+      mbar_init(smem_u32(&bars->tfull[h]), 1);
+      mbar_init(smem_u32(&bars->tempty[h]), F_EPI);
       mbar_init(smem_u32(&bars->done[h]), 1);
     }
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -259,20 +146,16 @@ __global__ void __launch_bounds__(F_THREADS, 1) k_assemble_fp64_tc(const Fp64Par
     const uint4* src = reinterpret_cast<const uint4*>(p.digits + (size_t)m0 * DG::SLICE);
     uint4* dst = reinterpret_cast<uint4*>(sA);
     for (int i = threadIdx.x; i < ms * (DG::SLICE / 16); i += F_THREADS) dst[i] = __ldg(src + i);
-    if constexpr (DG::BCH > ND * KC) {  // the chunk that pairs with the table's zero chunk
-      for (int i = threadIdx.x; i < F_HALVES * nst * FN; i += F_THREADS)
-        *reinterpret_cast<uint4*>(sB + (i / FN) * DG::STAGE + (ND * KC * FN + i % FN) * 16) = make_uint4(0, 0, 0, 0);
-    }
   }
   fence_proxy_async();
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
-  const uint32_t tmem = bars->tmem_base + half * (F_UNITS * 2 * FN);
+  const uint32_t tmem = bars->tmem_base + half * F_COLS;
   sB += half * nst * DG::STAGE;
   sX += half * F_XRING * FN;
   const uint32_t full = smem_u32(bars->full[half]), empty = smem_u32(bars->empty[half]);
-  const uint32_t tfull = smem_u32(bars->tfull[half]), tempty = smem_u32(bars->tempty[half]);
+  const uint32_t tfull = smem_u32(&bars->tfull[half]), tempty = smem_u32(&bars->tempty[half]);
 
   if (warp >= F_PWARP0 && warp < F_MWARP0) {
     // ---------------- producers: a tile per warp, a cell per thread ----------------
@@ -293,13 +176,15 @@ __global__ void __launch_bounds__(F_THREADS, 1) k_assemble_fp64_tc(const Fp64Par
       int X = 0;  // largest biased exponent of the scaled factors, in place (<< 20)
       if (!flag) {
         bool wild = false;
+        uint32_t some = 0;
 #pragma unroll
         for (int k = 0; k < K; ++k) {
+          some |= (uint32_t)__double2hiint(G[k]) << 1 | (uint32_t)__double2loint(G[k]);
           const int ef = __double2hiint(G[k]) & 0x7FF00000;
           wild = wild || ef == 0x7FF00000;
           if (ef != 0) X = max(X, ef + p.tk20[term_of<FORM, D>(k)]);
         }
-        wild = wild || (X != 0 && (X < (123 << 20) || X > (1923 << 20)));
+        wild = wild || (some != 0 && (X < (123 << 20) || X > (1923 << 20)));
         if (wild) flag = 2;
       }
       if (flag) {
@@ -322,7 +207,8 @@ __global__ void __launch_bounds__(F_THREADS, 1) k_assemble_fp64_tc(const Fp64Par
           U[j] = k < K ? fixed_point<DG::bias(), DG::FB>(G[k < K ? k : 0], X, p.tk20[term_of<FORM, D>(k < K ? k : 0)])
                        : DG::bias();
         }
-        store_digits<B, ND, KC>(dst, c, U, c == KC - 1);
+        if (c == KC - 1) store_digits<B, ND, FN * 16, true>(dst + c * (ND * FN * 16), U);
+        else store_digits<B, ND, FN * 16, false>(dst + c * (ND * FN * 16), U);
       }
       sX[(i % F_XRING) * FN + lane] = flag == 1 ? CELL_SKIP : flag == 2 ? CELL_PLAIN : X - (1022 << 20);
       fence_proxy_async();
@@ -330,46 +216,42 @@ __global__ void __launch_bounds__(F_THREADS, 1) k_assemble_fp64_tc(const Fp64Par
     }
   } else if (warp >= F_MWARP0) {
     // ---------------- MMA issuer ----------------
-    // The whole warp runs the loop, so that descriptors stay in uniform registers; one lane issues.
-    {
-      const uint32_t lead = lane == 0;
-      const uint32_t idesc = make_idesc(0, BM, FN);  // f16 operands
-      const uint64_t a0 = f_desc(smem_u32(sA), BM * 16), b0 = f_desc(smem_u32(sB), FN * 16);
-      uint32_t slice = 0;  // slices done: the parity of every unit
+    // Digit q of T against the cells' digits 0 .. ND-1-q at once: their 32-row blocks follow one another as
+    // the orders' columns do, so one MMA of N = 32 (ND - q) adds to the orders q .. ND-1. An MMA takes 45 cycles
+    // at N <= 64 and N / 2 from 128 on, its issue as long or longer, so few wide ones matter (advection-
+    // diffusion: 24 a slice of 128 entries where an MMA per pair of digits and two K chunks took 92).
+    if (lane == 0) {
+      const uint32_t a0 = smem_u32(sA), b0 = smem_u32(sB);
+      uint32_t slice = 0;
       int64_t i = 0;
       bool ok = true;
       for (int64_t t = t0; t < ntiles && ok; t += tstep, ++i) {
         const int s = (int)(i % nst);
         if (!mbar_wait(full + 8 * s, (uint32_t)((i / nst) & 1), p.err)) break;
         tc_fence_after();
-        const uint64_t bs = b0 + (uint32_t)(s * (DG::STAGE / 16));  // descriptor addresses count 16 bytes
-        for (int m = 0; m < ms && ok; ++m, ++slice) {
-          const uint64_t as = a0 + (uint32_t)(m * (DG::SLICE / 16));
+        for (int m = 0; m < ms; ++m, ++slice) {
+          if (!mbar_wait(tempty, (slice & 1u) ^ 1u, p.err)) { ok = false; break; }
+          tc_fence_after();
 #pragma unroll
-          for (int u = 0; u < F_UNITS; u += 2) {
-            if (!mbar_wait(tempty + 8 * u, (slice & 1u) ^ 1u, p.err) ||
-                !mbar_wait(tempty + 8 * u + 8, (slice & 1u) ^ 1u, p.err)) {
-              ok = false;
-              break;
+          for (int c = 0; c < KC; c += 2) {
+            // the last chunk of an odd number: the other half of the K step is the table's zero chunk, against
+            // which the cells' side may read any finite halves, here the table's
+            const bool odd = c == KC - 1;
+            const uint32_t bc = b0 + (uint32_t)(s * DG::STAGE + c * (ND * FN * 16));
+            const uint64_t bd = f_desc(bc, odd ? a0 - bc : ND * FN * 16);
+#pragma unroll
+            for (int q = 0; q < ND; ++q) {
+              const uint32_t chunk = (uint32_t)(q * KC + c);
+              const uint64_t ad = f_desc(a0 + (uint32_t)(m * DG::SLICE) + chunk * (BM * 16),
+                                         (odd ? (uint32_t)(ND * KC) - chunk : 1u) * (BM * 16));
+              mma<false>(tmem + q * FN, ad, bd, make_idesc(0, BM, (ND - q) * FN), c | q ? 1u : 0u);
             }
-            tc_fence_after();
-#pragma unroll
-            for (int q = 0; q < (KC * ND + 1) / 2; ++q)
-#pragma unroll
-              for (int w = 0; w < 4; ++w) {
-                const int d = 7 - 2 * u - w;
-                if (d >= ND || q >= (KC * (d + 1) + 1) / 2) continue;
-                constexpr int step_a = 2 * BM, step_b = 2 * FN;
-                f_mma(lead, tmem + u * 2 * FN + w * FN, as + (uint32_t)((ND - 1 - d) * KC * BM + q * step_a),
-                           bs + q * step_b, idesc, q ? 1u : 0u);
-              }
-            f_commit(lead, tfull + 8 * u);
-            f_commit(lead, tfull + 8 * u + 8);
           }
+          tc_commit(tfull);
         }
-        f_commit(lead, empty + 8 * s);
+        tc_commit(empty + 8 * s);
       }
-      f_commit(lead, smem_u32(&bars->done[half]));
+      tc_commit(smem_u32(&bars->done[half]));
       mbar_wait(smem_u32(&bars->done[half]), 0, p.err);
     }
     __syncwarp();
@@ -379,20 +261,11 @@ __global__ void __launch_bounds__(F_THREADS, 1) k_assemble_fp64_tc(const Fp64Par
     const uint32_t tcol = tmem + ((uint32_t)(q * 32) << 16) + sub * FC;
     uint32_t slice = 0;
     bool ok = true;
-    // unit u's accumulators: order 7 - 2 u (where there is one) and order 6 - 2 u
-    auto load = [&](int u, uint32_t (&r0)[FC], uint32_t (&r1)[FC], bool both) {
-      if (!mbar_wait(tfull + 8 * u, slice & 1u, p.err)) return false;
-      __syncwarp();
-      tc_fence_after();
-      if (both) tmem_ld16(tcol + u * 2 * FN, r0);
-      tmem_ld16(tcol + u * 2 * FN + FN, r1);
+    // the accumulators of orders d and d - 1 (r0, r1), of the latter alone with both = false
+    auto load = [&](int d, uint32_t (&r0)[FC], uint32_t (&r1)[FC], bool both) {
+      if (both) tmem_ld16(tcol + d * FN, r0);
+      tmem_ld16(tcol + (d - 1) * FN, r1);
       tmem_wait_ld();
-      return true;
-    };
-    auto release = [&](int u) {
-      tc_fence_before();
-      __syncwarp();
-      if (lane == 0) mbar_arrive(tempty + 8 * u);
     };
     const uint32_t pB = opaque(1u << B), pB4 = opaque(1u << (B + 4)), p4 = opaque(16u), p18 = opaque(1u << 18),
                    p20 = opaque(1u << 20), p22 = opaque(1u << 22);
@@ -412,15 +285,16 @@ __global__ void __launch_bounds__(F_THREADS, 1) k_assemble_fp64_tc(const Fp64Par
         uint32_t lo[FC], hi[FC];
         {
           uint32_t r0[FC], r1[FC];
-          if (!(ok = load(0, r0, r1, B == 8))) break;  // orders 7 (b = 8, without the constant) and 6
-          release(0);
+          if (!mbar_wait(tfull, slice & 1u, p.err)) { ok = false; break; }
+          __syncwarp();
+          tc_fence_after();
+          load(7, r0, r1, B == 8);  // orders 7 (b = 8, without the constant) and 6
 #pragma unroll
           for (int j = 0; j < FC; ++j)
             lo[j] = B == 9 ? r1[j] >> 9
                            : (r1[j] >> 4) + (__float_as_uint(__uint_as_float(r0[j]) + 25165824.0f) >> 11) +
                                  (0x4C000000u - (MAGIC >> 4) - (0x4BC00000u >> 11));
-          if (!(ok = load(1, r0, r1, true))) break;  // orders 5, 4
-          release(1);
+          load(5, r0, r1, true);
 #pragma unroll
           for (int j = 0; j < FC; ++j) {
             const uint32_t c = mad_lo(r1[j], pB, r0[j]);
@@ -432,8 +306,7 @@ __global__ void __launch_bounds__(F_THREADS, 1) k_assemble_fp64_tc(const Fp64Par
               hi[j] = (uint32_t)(S >> 32);
             }
           }
-          if (!(ok = load(2, r0, r1, true))) break;  // orders 3, 2
-          release(2);
+          load(3, r0, r1, true);
 #pragma unroll
           for (int j = 0; j < FC; ++j) {
             const uint64_t S =
@@ -450,18 +323,15 @@ __global__ void __launch_bounds__(F_THREADS, 1) k_assemble_fp64_tc(const Fp64Par
 #pragma unroll
           for (int j = 0; j < FC; ++j) pos[j] = o < N && cbase + j < p.ncells ? __ldg(mp + j * bw) : 0xffffffffu;
         }
-        // orders 1 and 0: the high word alone (one at a time, for the registers)
-        if (!mbar_wait(tfull + 24, slice & 1u, p.err)) { ok = false; break; }
-        __syncwarp();
-        tc_fence_after();
+        // orders 1 and 0: the high word alone
+        {
+          uint32_t r0[FC], r1[FC];
+          load(1, r0, r1, true);
+          tc_fence_before();
+          __syncwarp();
+          if (lane == 0) mbar_arrive(tempty);
 #pragma unroll
-        for (int w = 0; w < 2; ++w) {
-          uint32_t r[FC];
-          tmem_ld16(tcol + 3 * 2 * FN + w * FN, r);
-          tmem_wait_ld();
-          if (w == 1) release(3);
-#pragma unroll
-          for (int j = 0; j < FC; ++j) hi[j] = mad_lo(r[j], w ? pB4 : p4, hi[j]);
+          for (int j = 0; j < FC; ++j) hi[j] = mad_lo(r1[j], pB4, mad_lo(r0[j], p4, hi[j]));
         }
         if ((m0 + m) * BM + q * 32 >= N) continue;  // warp-uniform
         const int* xs = sX + (i % F_XRING) * FN + sub * FC;
@@ -558,15 +428,6 @@ cudaError_t launch_digits(const Fp64Params& p, int num_sms, cudaStream_t s) {
   return cudaGetLastError();
 }
 
-uint16_t half_of_int(int v) {  // |v| <= 4096, exact in a half
-  if (v == 0) return 0;
-  const uint16_t s = v < 0 ? 0x8000 : 0;
-  unsigned a = (unsigned)std::abs(v);
-  int e = 0;
-  while ((a >> e) > 1) ++e;
-  return (uint16_t)(s | ((e + 15) << 10) | ((e <= 10 ? a << (10 - e) : a >> (e - 10)) & 0x3FFu));
-}
-
 template <int FORM, int D>
 void image_of(int degree, int cell, std::vector<uint8_t>& img, std::vector<int32_t>& y20, int32_t (&tk20)[2]) {
   using DG = Digits<FORM, D>;
@@ -596,7 +457,7 @@ void image_of(int degree, int cell, std::vector<uint8_t>& img, std::vector<int32
     y20[o] = (y - (DG::B == 9 ? 59 : 56) + 1054) * (1 << 20);
     uint8_t* slice = img.data() + (size_t)(o / BM) * DG::SLICE + (size_t)(o % BM) * 16;
     for (int q = 0; q < DG::ND; ++q) {
-      const int block = (DG::ND - 1 - q) * DG::KC;  // digit q counts from the leading one
+      const int block = q * DG::KC;  // digit q counts from the leading one
       for (int k = 0; k < DG::K; ++k) {
         const double f = std::nearbyint(std::ldexp(T[(size_t)k * N + o], DG::FB - tk[term_of<FORM, D>(k)] - y));
         const uint64_t U = (uint64_t)(int64_t)f + DG::bias();
@@ -616,7 +477,7 @@ void image_of(int degree, int cell, std::vector<uint8_t>& img, std::vector<int32
 }  // namespace
 
 // Where the digit contraction runs instead of the plain kernel: where it is the faster one at every count
-// of cells, from 300 (both launch-bound, 8-20 us against 11-2300 us) to 196,608 (53-1434 us against
+// of cells, from 300 (both launch-bound, 8-20 us against 11-2300 us) to 196,608 (53-1100 us against
 // 84-16,900 us). Left to the plain kernel are P1 triangles (9 entries: Helmholtz 32 against 47 us) and the
 // mass matrices of up to 6 nodes (one multiplication an entry: P2 triangles at 300 cells 5 against 9 us).
 int fp64_tc_use(int form, int degree, int cell) {
