@@ -135,7 +135,7 @@ struct TcEntry {
 
 struct DigitEntry {
   uint8_t* image = nullptr;
-  int32_t* y20 = nullptr;
+  int32_t* exps = nullptr;
   int32_t tk20[2] = {0, 0};
 };
 
@@ -144,7 +144,7 @@ struct DeviceCache {
   int num_sms = 0;
   std::map<std::tuple<int, int, int>, double*> fp64;    // (form, degree, cell)
   std::map<std::tuple<int, int, int, int>, TcEntry> tc;  // + precision
-  std::map<std::tuple<int, int, int>, DigitEntry> digits;  // FP64 on the tensor cores
+  std::map<std::tuple<int, int, int>, DigitEntry> digits, adjoint;  // FP64 on the tensor cores
 };
 
 std::mutex g_mu;
@@ -202,6 +202,22 @@ int fp64_table(DeviceCache& c, int form, int degree, int cell, const double** T)
   return COFFEE_OK;
 }
 
+// image followed by 32-bit exponents, uploaded as one allocation
+int upload_digits(std::vector<uint8_t>& img, const std::vector<int32_t>& exps, DigitEntry& ent) {
+  const size_t at = (img.size() + 15) & ~size_t(15), bytes = at + exps.size() * sizeof(int32_t);
+  img.resize(bytes);
+  std::memcpy(img.data() + at, exps.data(), exps.size() * sizeof(int32_t));
+  cudaError_t e = cudaMalloc(&ent.image, bytes);
+  if (e != cudaSuccess) return cuda_fail(e, "cudaMalloc(digit table)");
+  e = cudaMemcpy(ent.image, img.data(), bytes, cudaMemcpyHostToDevice);
+  if (e != cudaSuccess) {
+    cudaFree(ent.image);
+    return cuda_fail(e, "cudaMemcpy(digit table)");
+  }
+  ent.exps = reinterpret_cast<int32_t*>(ent.image + at);
+  return COFFEE_OK;
+}
+
 int digit_table(DeviceCache& c, int form, int degree, int cell, Fp64Params& p) {
   auto key = std::make_tuple(form, degree, cell);
   auto it = c.digits.find(key);
@@ -210,23 +226,31 @@ int digit_table(DeviceCache& c, int form, int degree, int cell, Fp64Params& p) {
     std::vector<int32_t> y20;
     DigitEntry ent;
     build_fp64_image(form, degree, cell, img, y20, ent.tk20);
-    const size_t at = (img.size() + 15) & ~size_t(15), bytes = at + y20.size() * sizeof(int32_t);
-    img.resize(bytes);
-    std::memcpy(img.data() + at, y20.data(), y20.size() * sizeof(int32_t));
-    cudaError_t e = cudaMalloc(&ent.image, bytes);
-    if (e != cudaSuccess) return cuda_fail(e, "cudaMalloc(digit table)");
-    e = cudaMemcpy(ent.image, img.data(), bytes, cudaMemcpyHostToDevice);
-    if (e != cudaSuccess) {
-      cudaFree(ent.image);
-      return cuda_fail(e, "cudaMemcpy(digit table)");
-    }
-    ent.y20 = reinterpret_cast<int32_t*>(ent.image + at);
+    int rc = upload_digits(img, y20, ent);
+    if (rc != COFFEE_OK) return rc;
     it = c.digits.emplace(key, ent).first;
   }
   p.digits = it->second.image;
-  p.yexp20 = it->second.y20;
+  p.yexp20 = it->second.exps;
   p.tk20[0] = it->second.tk20[0];
   p.tk20[1] = it->second.tk20[1];
+  return COFFEE_OK;
+}
+
+int adjoint_table(DeviceCache& c, int form, int degree, int cell, BwdParams& p) {
+  auto key = std::make_tuple(form, degree, cell);
+  auto it = c.adjoint.find(key);
+  if (it == c.adjoint.end()) {
+    std::vector<uint8_t> img;
+    std::vector<int32_t> kexp20;
+    DigitEntry ent;
+    build_backward_image(form, degree, cell, img, kexp20);
+    int rc = upload_digits(img, kexp20, ent);
+    if (rc != COFFEE_OK) return rc;
+    it = c.adjoint.emplace(key, ent).first;
+  }
+  p.digits = it->second.image;
+  p.kexp20 = it->second.exps;
   return COFFEE_OK;
 }
 
@@ -715,8 +739,19 @@ int coffee_assemble_backward(const coffee_assemble_args* a, const void* dout, do
   p.N = ns * ns;
   p.validate = (a->flags & COFFEE_FLAG_VALIDATE) ? 1 : 0;
   cudaStream_t s = stream;
+  // FP64: the digit contraction on the tensor cores, unless the CUDA cores are asked for; not for the
+  // deterministic adjoint of few cells, whose results the allocation-free entry point repeats bit for bit
+  // (it has no memory for the digit table)
+  const bool digits = a->precision == PREC_FP64 && !(a->flags & COFFEE_FLAG_CUDA_CORES) &&
+                      backward_tc_use(a->form, a->degree, a->cell) &&
+                      !(deterministic && a->ncells <= NOALLOC_MAX_CELLS);
+  if (digits && (rc = adjoint_table(*c, a->form, a->degree, a->cell, p)) != COFFEE_OK) return rc;
+  auto launch = [&]() {
+    return (cudaError_t)(digits ? launch_backward_tc(a->form, a->cell, p, c->num_sms, s)
+                                : launch_backward(a->form, a->cell, p, s));
+  };
   if (!deterministic) {
-    cudaError_t e = (cudaError_t)launch_backward(a->form, a->cell, p, s);
+    cudaError_t e = launch();
     if (e != cudaSuccess) return cuda_fail(e, "launch(assemble_backward)");
     return COFFEE_OK;
   }
@@ -740,7 +775,7 @@ int coffee_assemble_backward(const coffee_assemble_args* a, const void* dout, do
   int64_t* off = reinterpret_cast<int64_t*>(ws + al(b_local) + 2 * al(b_cnt));
   int64_t* slots = reinterpret_cast<int64_t*>(ws + al(b_local) + 2 * al(b_cnt) + al(b_off));
   p.local = local;
-  e = (cudaError_t)launch_backward(a->form, a->cell, p, s);
+  e = launch();
   if (e == cudaSuccess)
     e = (cudaError_t)launch_ordered_sum(a->cell2vert, a->ncells, (int)width, a->nverts, local, nl, 0, d,
                                         d_coords, d, 0, cnt, cur, off, slots, c->err, s);

@@ -55,6 +55,8 @@ void prism_burgers_table(int k, std::vector<double>& tab, int& Q);
 
 // ---- error reporting (api.cu) ----
 int fail(int status, const std::string& msg);
+// cells the allocation-free adjoint takes at most (noalloc.cu)
+constexpr int64_t NOALLOC_MAX_CELLS = 16384;
 // the allocation-free adjoint's own error word on the current device, read and cleared (noalloc.cu)
 int noalloc_error_word(unsigned* w);
 
@@ -128,7 +130,13 @@ struct BwdParams {
   int64_t ncells, nverts, ncoefnodes;
   int N;
   int validate;
+  const uint8_t* digits;  // tensor-core kernel: digit image of T and the factors' exponents (<< 20)
+  const int32_t* kexp20;
 };
+// FP64 adjoint on the tensor cores by exact digit products (k_bwd_tc.cu)
+int backward_tc_use(int form, int degree, int cell);
+void build_backward_image(int form, int degree, int cell, std::vector<uint8_t>& img, std::vector<int32_t>& kexp20);
+int launch_backward_tc(int form, int cell, const BwdParams& p, int num_sms, void* stream);
 int bwd_local_len(int form, int cell);
 int launch_backward(int form, int cell, const BwdParams& p, void* stream);
 int launch_ordered_sum(const int32_t* idx, int64_t ncells, int width, int64_t nnodes, const double* local,

@@ -28,7 +28,6 @@
 namespace coffee {
 namespace {
 
-constexpr int64_t NOALLOC_MAX_CELLS = 16384;
 constexpr int64_t NOALLOC_MAX_NODES = 16384;
 constexpr int NL_MAX = 28;              // longest per-cell gradient: advection-diffusion on tets
 constexpr int64_t T_MAX = 36 * 1225;    // largest FP64 reference tensor: advection-diffusion, tet P4
