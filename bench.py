@@ -233,6 +233,20 @@ def alg_bytes_per_cell(wl, mesh, c2d, coef, ndof, out_bytes):
     return b
 
 
+def prism_fma(form, k):
+    """FP64 FMAs of one prism: per point the geometry and factors (about 60, Burgers also u from the triangle's
+    functions), then the sums over z (per triangle point and pair of z functions) and over the triangle's
+    points (per pair of z and pair of triangle functions; residual: per function)."""
+    burgers = form in (BURGERS_JAC, BURGERS_RESIDUAL)
+    p, nt, nz = ((3 * k + 3) // 2 if burgers else k + 2), (k + 1) * (k + 2) // 2, k + 1
+    point = p ** 3 * (60 + (12 * nt if burgers else 0))
+    if form == BURGERS_RESIDUAL:
+        return point + p ** 3 * nz * 12 + p * p * nt * nz * 9
+    ntp, nzp = nt * (nt + 1) // 2, nz * (nz + 1) // 2
+    fields, per = {MASS: (1, 1), HELMHOLTZ: (9, 13), ADVDIFF: (12, 18), BURGERS_JAC: (21, 27)}[form]
+    return point + p ** 3 * nzp * fields + p * p * ntp * nzp * per
+
+
 class ClockSampler:
     """nvidia-smi clocks and throttle reasons sampled every 100 ms during the timed region."""
 
@@ -554,12 +568,8 @@ def run_ours(args):
                         "by coffee_peak_fp64), the digit products on the tensor cores by their integer epilogue"
                         % device_peaks(coffee)["fp64_tflops"])
     if cell == PRISM and form in (BURGERS_JAC, BURGERS_RESIDUAL):
-        # vector Burgers, evaluated point by point: per point the factors (u, grad u, K: about 12
-        # FMAs per node and component set) and, per scalar pair (i, j), 9 FMAs for the component
-        # blocks and 12 for the diagonal terms (residual: 12 per node)
-        Q = ((3 * degree + 3) // 2) ** 3
-        n = ndof // 3
-        fma = Q * (12 * n + 60 + (12 * n if form == BURGERS_RESIDUAL else 21 * n * n))
+        # vector Burgers in FP64: the FMAs of the sums taken direction by direction
+        fma = prism_fma(form, degree)
         tf = 2.0 * fma * ncells / (launch_ms / 1e3) / 1e12
         p64 = device_peaks(coffee)["fp64_tflops"]
         roof = {"bound": "alu", "achieved": tf, "peak": p64, "unit": "TFLOP/s", "frac": tf / p64, "traffic": None,
@@ -571,6 +581,7 @@ def run_ours(args):
         K = Q * {HELMHOLTZ: 7, ADVDIFF: 9}.get(form, 1)
         flops = 2.0 * K * ndof * ndof + 250.0 * Q  # algorithmic, per cell
         if prec == coffee.FP64:
+            flops = 2.0 * prism_fma(form, degree)
             tf = flops * ncells / (launch_ms / 1e3) / 1e12
             p64 = device_peaks(coffee)["fp64_tflops"]
             roof = {"bound": "alu", "achieved": tf, "peak": p64, "unit": "TFLOP/s",

@@ -176,16 +176,8 @@ int fp64_table(DeviceCache& c, int form, int degree, int cell, const double** T)
     return COFFEE_OK;
   }
   std::vector<double> h;
-  if (cell == CELL_PRISM && form == FORM_BURGERS) {
-    // the basis at the Burgers rule's points, then the points and weights
-    int Q = 0;
-    prism_burgers_table(degree, h, Q);
-  } else if (cell == CELL_PRISM) {
-    // per-point tensors, then the rule's points and weights (read by the prism kernel)
-    std::vector<double> pts, wts;
-    prism_tensor(form, degree, h, pts, wts);
-    h.insert(h.end(), pts.begin(), pts.end());
-    h.insert(h.end(), wts.begin(), wts.end());
+  if (cell == CELL_PRISM) {
+    prism_sum_table(form, degree, h);
   } else {
     reference_tensor(form, degree, cell, h);
   }
@@ -348,11 +340,11 @@ int assemble_impl(const coffee_assemble_args* a, const uint32_t* map, int64_t nn
     if (e != cudaSuccess) return cuda_fail(e, ("launch(assemble_prism_tc) " + why).c_str());
     return COFFEE_OK;
   }
-  if (a->cell == CELL_PRISM && burgers_like(a->form)) {
+  if (a->cell == CELL_PRISM) {
     if (map && a->form == FORM_BURGERS_RES) return fail(COFFEE_ERR_UNSUPPORTED, "global assembly of element vectors");
     const double* T = nullptr;
     if ((rc = fp64_table(*c, a->form, a->degree, a->cell, &T)) != COFFEE_OK) return rc;
-    const int pb = prism_burgers_points(a->degree);
+    const int points = prism_points(a->form, a->degree);
     PrismParams p{};
     p.coords = a->coords;
     p.c2v = a->cell2vert;
@@ -364,39 +356,12 @@ int assemble_impl(const coffee_assemble_args* a, const uint32_t* map, int64_t nn
     p.err = c->err;
     p.ncells = a->ncells;
     p.nverts = a->nverts;
-    p.Q = pb * pb * pb;
-    p.N = prism_nnodes(a->degree);
+    p.Q = points * points * points;
     p.validate = validate ? 1 : 0;
     p.nu = a->nu;
     p.map = map;
     p.nnz = nnz;
-    cudaError_t e = (cudaError_t)launch_prism_burgers(a->form, a->degree, p, c->num_sms, stream);
-    if (e != cudaSuccess) return cuda_fail(e, "launch(prism_burgers)");
-    return COFFEE_OK;
-  }
-  if (a->cell == CELL_PRISM) {
-    if (!(a->form == FORM_MASS || a->form == FORM_HELMHOLTZ || a->form == FORM_ADVDIFF))
-      return fail(COFFEE_ERR_UNSUPPORTED, "prisms: MASS, HELMHOLTZ and ADVDIFF");
-    const double* T = nullptr;
-    if ((rc = fp64_table(*c, a->form, a->degree, a->cell, &T)) != COFFEE_OK) return rc;
-    const int n = prism_nnodes(a->degree);
-    PrismParams p{};
-    p.coords = a->coords;
-    p.c2v = a->cell2vert;
-    p.coef = a->coef;
-    p.c2d = a->cell2dof;
-    p.ncoefnodes = a->ncoefnodes;
-    p.T = T;
-    p.out = a->out;
-    p.err = c->err;
-    p.ncells = a->ncells;
-    p.nverts = a->nverts;
-    p.Q = (a->degree + 2) * (a->degree + 2) * (a->degree + 2);
-    p.N = n * n;
-    p.validate = validate ? 1 : 0;
-    p.map = map;
-    p.nnz = nnz;
-    cudaError_t e = (cudaError_t)launch_prism(a->form, p, c->num_sms, stream);
+    cudaError_t e = (cudaError_t)launch_prism(a->form, a->degree, p, c->num_sms, stream);
     if (e != cudaSuccess) return cuda_fail(e, "launch(assemble_prism)");
     return COFFEE_OK;
   }

@@ -50,8 +50,8 @@ void prism_rule(int k, std::vector<double>& pts, std::vector<double>& wts);
 void prism_basis(int k, int npts, const double* x, double* phi, double* grads);
 void prism_tensor(int form, int k, std::vector<double>& T, std::vector<double>& pts, std::vector<double>& wts);
 void prism_rule_points(int n, std::vector<double>& pts, std::vector<double>& wts);
-int prism_burgers_points(int k);
-void prism_burgers_table(int k, std::vector<double>& tab, int& Q);
+int prism_points(int form, int k);
+void prism_sum_table(int form, int k, std::vector<double>& tab);
 
 // ---- error reporting (api.cu) ----
 int fail(int status, const std::string& msg);
@@ -88,27 +88,24 @@ void build_fp64_image(int form, int degree, int cell, std::vector<uint8_t>& img,
                       int32_t (&tk20)[2]);
 int launch_fp64_tc(int form, int cell, const Fp64Params& p, int num_sms, void* stream);
 
-// ---- FP64 prism kernel (k_prism.cu) ----
+// ---- FP64 prism kernels (k_prism_sf.cu) ----
 struct PrismParams {
   const double* coords;  // [nverts][3]
   const int32_t* c2v;    // [ncells][6]
-  const double* coef;    // ADVDIFF: rows (eps, b0, b1, b2) per coefficient node
-  const int32_t* c2d;    // ADVDIFF: [ncells][6]
+  const double* coef;    // ADVDIFF: rows (eps, b0, b1, b2) per coefficient node; Burgers: u [ncoefnodes][3]
+  const int32_t* c2d;    // ADVDIFF: [ncells][6]; Burgers: [ncells][n]
   int64_t ncoefnodes;
-  const double* T;       // [Q*KQ][N] per-point tensors, then points [Q][3], then weights [Q]
-  void* out;             // double [ncells][N], or the CSR values when map is set
+  const double* T;       // prism_sum_table
+  void* out;             // double [ncells][N][N] or [ncells][N], or the CSR values when map is set
   unsigned* err;
   int64_t ncells, nverts;
-  int Q, N;
+  int Q;                 // points
   int validate;
   const uint32_t* map;   // global assembly (blocked entry map), else NULL
   int64_t nnz;
   double nu;             // Burgers viscosity
 };
-int launch_prism(int form, const PrismParams& p, int num_sms, void* stream);
-// vector Burgers on prisms, FP64 (k_prism_burgers.cu): the Jacobian (FORM_BURGERS) or the residual
-// (FORM_BURGERS_RES); p.T holds prism_burgers_table, p.N the nodes n of one component, p.Q points
-int launch_prism_burgers(int form, int degree, const PrismParams& p, int num_sms, void* stream);
+int launch_prism(int form, int degree, const PrismParams& p, int num_sms, void* stream);
 // tensor-core prisms (k_prism_tc.cu): K-chunked streamed contraction, MASS/HELMHOLTZ/ADVDIFF P1-P4
 struct TcParams;
 struct TcTable;

@@ -286,6 +286,18 @@ void prism_rule_points(int n, std::vector<double>& pts, std::vector<double>& wts
 
 void prism_rule(int k, std::vector<double>& pts, std::vector<double>& wts) { prism_rule_points(k + 2, pts, wts); }
 
+// Interval Lagrange function c on the nodes m/k at z, prod_{m != c} (k z - m) / (c - m), and its derivative
+static void interval_basis(int k, int c, double z, double& L, double& dL) {
+  L = 1.0;
+  dL = 0.0;
+  for (int m = 0; m <= k; ++m) {
+    if (m == c) continue;
+    const double f = (k * z - m) / (double)(c - m), df = k / (double)(c - m);
+    dL = dL * f + L * df;
+    L *= f;
+  }
+}
+
 void prism_basis(int k, int npts, const double* x, double* phi, double* grads) {
   const int nt = (k + 1) * (k + 2) / 2, n = prism_nnodes(k);
   std::vector<double> tp(nt), tg((size_t)nt * 2);
@@ -293,14 +305,8 @@ void prism_basis(int k, int npts, const double* x, double* phi, double* grads) {
     const double* xp = x + (size_t)p * 3;
     lagrange_basis(0, k, 1, xp, tp.data(), tg.data());
     for (int c = 0; c <= k; ++c) {
-      // interval Lagrange function on the nodes m/k: prod_{m != c} (k z - m) / (c - m)
-      double L = 1.0, dL = 0.0;
-      for (int m = 0; m <= k; ++m) {
-        if (m == c) continue;
-        const double f = (k * xp[2] - m) / (double)(c - m), df = k / (double)(c - m);
-        dL = dL * f + L * df;
-        L *= f;
-      }
+      double L, dL;
+      interval_basis(k, c, xp[2], L, dL);
       for (int t = 0; t < nt; ++t) {
         const size_t i = (size_t)p * n + (size_t)c * nt + t;
         if (phi) phi[i] = tp[t] * L;
@@ -350,26 +356,61 @@ void prism_tensor(int form, int k, std::vector<double>& T, std::vector<double>& 
   }
 }
 
-// Vector Burgers on prisms: the basis at the points of its rule, (3k+3)/2 Gauss-Legendre points per
-// direction (the trilinear term phi_i phi_j grad u has degree 3k-1 in the triangle variables and
-// 3k in zeta on prisms with planar faces), as tab [Q][n][4] = (phi, d_s phi, d_t phi, d_z phi),
-// then the points [Q][3] and the weights [Q]. The kernel evaluates the quadrature loop directly.
-int prism_burgers_points(int k) { return (3 * k + 3) / 2; }
+// Points per direction of the FP64 prism kernels: the forms' rule, and for vector Burgers (3k+3)/2 (the
+// trilinear term phi_i phi_j grad u has degree 3k-1 in the triangle variables and 3k in zeta on prisms with
+// planar faces).
+int prism_points(int form, int k) { return burgers_like(form) ? (3 * k + 3) / 2 : k + 2; }
 
-void prism_burgers_table(int k, std::vector<double>& tab, int& Q) {
-  std::vector<double> pts, wts;
-  prism_rule_points(prism_burgers_points(k), pts, wts);
-  Q = (int)wts.size();
-  const int n = prism_nnodes(k);
-  std::vector<double> phi((size_t)Q * n), g((size_t)Q * n * 3);
-  prism_basis(k, Q, pts.data(), phi.data(), g.data());
-  tab.assign((size_t)Q * n * 4, 0.0);
-  for (size_t i = 0; i < (size_t)Q * n; ++i) {
-    tab[i * 4] = phi[i];
-    for (int a = 0; a < 3; ++a) tab[i * 4 + 1 + a] = g[i * 3 + a];
-  }
-  tab.insert(tab.end(), pts.begin(), pts.end());
-  tab.insert(tab.end(), wts.begin(), wts.end());
+// Tables of the direction-by-direction sums over a prism's points (p per direction; qt over the triangle's
+// p^2, qz over z's p), nt triangle and k+1 interval functions, pairs (i <= j) numbered j (j+1)/2 + i:
+//   [qt][nt][3]      psi, d_s psi, d_t psi
+//   [qt][8][pairs]   psi_i psi_j; the d_s d_s, (d_s d_t + d_t d_s), d_t d_t products; d_s psi_i psi_j, psi_i d_s psi_j;
+//                    the same with d_t
+//   [qz][pairs][4]   zeta_i zeta_j, zeta_i zeta'_j, zeta_j zeta'_i, zeta'_i zeta'_j
+//   [qz][k+1][2]     zeta, zeta'
+//   [qt][3], [qz][2] points and weights (s, t, weight), (z, weight)
+void prism_sum_table(int form, int k, std::vector<double>& tab) {
+  const int p = prism_points(form, k), nt = (k + 1) * (k + 2) / 2;
+  std::vector<double> g, w;
+  gauss_jacobi01(p, 0, g, w);
+  std::vector<double> psi((size_t)p * p * nt), dpsi((size_t)p * p * nt * 2), zeta((size_t)p * (k + 1) * 2);
+  tab.clear();
+  for (int i = 0; i < p; ++i)
+    for (int j = 0; j < p; ++j) {
+      const int qt = i * p + j;
+      const double x[2] = {g[i], g[j] * (1.0 - g[i])};
+      lagrange_basis(0, k, 1, x, &psi[(size_t)qt * nt], &dpsi[(size_t)qt * nt * 2]);
+      for (int t = 0; t < nt; ++t) {
+        tab.push_back(psi[(size_t)qt * nt + t]);
+        tab.push_back(dpsi[((size_t)qt * nt + t) * 2]);
+        tab.push_back(dpsi[((size_t)qt * nt + t) * 2 + 1]);
+      }
+    }
+  for (int qt = 0; qt < p * p; ++qt)
+    for (int kind = 0; kind < 8; ++kind)
+      for (int j = 0; j < nt; ++j)
+        for (int i = 0; i <= j; ++i) {
+          const double a = psi[(size_t)qt * nt + i], b = psi[(size_t)qt * nt + j];
+          const double *da = &dpsi[((size_t)qt * nt + i) * 2], *db = &dpsi[((size_t)qt * nt + j) * 2];
+          const double v[8] = {a * b,     da[0] * db[0], da[0] * db[1] + da[1] * db[0], da[1] * db[1],
+                               da[0] * b, a * db[0],     da[1] * b,                     a * db[1]};
+          tab.push_back(v[kind]);
+        }
+  for (int q = 0; q < p; ++q)
+    for (int c = 0; c <= k; ++c)
+      interval_basis(k, c, g[q], zeta[((size_t)q * (k + 1) + c) * 2], zeta[((size_t)q * (k + 1) + c) * 2 + 1]);
+  for (int q = 0; q < p; ++q)
+    for (int j = 0; j <= k; ++j)
+      for (int i = 0; i <= j; ++i) {
+        const double *a = &zeta[((size_t)q * (k + 1) + i) * 2], *b = &zeta[((size_t)q * (k + 1) + j) * 2];
+        for (double v : {a[0] * b[0], a[0] * b[1], b[0] * a[1], a[1] * b[1]}) tab.push_back(v);
+      }
+  tab.insert(tab.end(), zeta.begin(), zeta.end());
+  for (int i = 0; i < p; ++i)
+    for (int j = 0; j < p; ++j)
+      for (double v : {g[i], g[j] * (1.0 - g[i]), w[i] * w[j] * (1.0 - g[i])}) tab.push_back(v);
+  for (int q = 0; q < p; ++q)
+    for (double v : {g[q], w[q]}) tab.push_back(v);
 }
 
 }  // namespace coffee
