@@ -140,6 +140,7 @@ struct DigitEntry {
 };
 
 struct DeviceCache {
+  std::map<std::tuple<int, int, int, int>, uint8_t*> shift;  // T^T of the sector-aligned stores
   unsigned* err = nullptr;
   int num_sms = 0;
   std::map<std::tuple<int, int, int>, double*> fp64;    // (form, degree, cell)
@@ -264,6 +265,26 @@ int tc_table(DeviceCache& c, int form, int degree, int cell, int prec, TcTable* 
     it = c.tc.emplace(key, ent).first;
   }
   *meta = it->second.meta;
+  return COFFEE_OK;
+}
+
+int shift_table(DeviceCache& c, int form, int degree, int cell, int prec, const uint8_t** image) {
+  auto key = std::make_tuple(form, degree, cell, prec);
+  auto it = c.shift.find(key);
+  if (it == c.shift.end()) {
+    std::vector<uint8_t> img;
+    build_shift_image(form, degree, cell, prec, img);
+    uint8_t* d = nullptr;
+    cudaError_t e = cudaMalloc(&d, img.size());
+    if (e != cudaSuccess) return cuda_fail(e, "cudaMalloc(shifted table)");
+    e = cudaMemcpy(d, img.data(), img.size(), cudaMemcpyHostToDevice);
+    if (e != cudaSuccess) {
+      cudaFree(d);
+      return cuda_fail(e, "cudaMemcpy(shifted table)");
+    }
+    it = c.shift.emplace(key, d).first;
+  }
+  *image = it->second;
   return COFFEE_OK;
 }
 
@@ -453,6 +474,9 @@ int assemble_impl(const coffee_assemble_args* a, const uint32_t* map, int64_t nn
     if (e != cudaSuccess) return cuda_fail(e, ("launch(assemble_simt) " + why).c_str());
     return COFFEE_OK;
   }
+  if (!map && tc_shift_use(a->form, a->degree, a->cell, a->precision, p.ostride, p.tune, a->ncells) &&
+      (rc = shift_table(*c, a->form, a->degree, a->cell, a->precision, &p.shift_image)) != COFFEE_OK)
+    return rc;
   cudaError_t e = map ? (cudaError_t)launch_tc_csr(a->form, a->cell, p, c->num_sms, stream, why)
                       : (cudaError_t)launch_tc(a->form, a->cell, p, c->num_sms, stream, why);
   if (e != cudaSuccess)

@@ -178,6 +178,8 @@ struct TcParams {
   int mtiles, kbytes, tparts;  // tparts: TcTable::tparts
   int ksteps_off;        // Burgers: K-steps of the off-diagonal component blocks
   unsigned tune;         // TUNE_* knobs
+  const uint8_t* shift_image;  // T^T for the sector-aligned stores (build_shift_image), or NULL
+  int classes;           // offsets of a row within a 32-byte sector (8 / gcd(ostride, 8)) when those are used
   int subw;              // cells per TMEM accumulator (outputs-on-lanes orientation)
   int stage_cells;       // staged epilogue: rows per bulk copy (0: direct stores)
   int stage_bufs;        // staged epilogue: buffers of stage_cells rows (2 to 4)
@@ -198,6 +200,11 @@ int tc_supported(int form, int degree, int cell, int precision);
 int staged_plan(const TcParams& p, int& subw, int& cells, int& buf_bytes);
 int launch_tc_staged(int form, int cell, const TcParams& q, int num_sms, void* stream, int nst, int smem);
 int launch_tc(int form, int cell, const TcParams& p, int num_sms, void* stream, std::string& why);
+// sector-aligned stores (k_tc_shift.cu): whether element matrices of this form, stride and precision take them, and the
+// image of T^T that they need (per part, 16-byte K chunk and row: 8 zero rows, then the outputs)
+int tc_shift_use(int form, int degree, int cell, int precision, int64_t ostride, unsigned tune, int64_t ncells);
+void build_shift_image(int form, int degree, int cell, int precision, std::vector<uint8_t>& img);
+int launch_tc_shift(int form, int cell, const TcParams& p, int num_sms, void* stream);
 // T [K][N] (FP64) of the tensor-core contraction: the stiffness tensors in the edge basis
 void tc_reference_tensor(int form, int degree, int cell, std::vector<double>& T);
 // CUDA-core kernel for small element matrices (k_simt.cu): MASS, HELMHOLTZ and ADVDIFF on

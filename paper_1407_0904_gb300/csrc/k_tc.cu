@@ -160,6 +160,7 @@ int launch_tc(int form, int cell, const TcParams& p, int num_sms, void* stream, 
   if (p.ncells == 0) return (int)cudaSuccess;
   if (form == FORM_BURGERS) return launch_burgers_tc(cell, p, num_sms, stream, why);
   if (form == FORM_BURGERS_RES) return launch_burgers_res_tc(cell, p, num_sms, stream, why);
+  if (p.shift_image != nullptr) return launch_tc_shift(form, cell, p, num_sms, stream);
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   Geom g{};
   g.kbytes = p.kbytes;

@@ -95,6 +95,11 @@ __device__ __forceinline__ uint64_t make_desc(uint32_t saddr, uint32_t sbo) {
   d |= 1ull << 46;  // descriptor version of tcgen05
   return d;
 }
+// The same with the distance lbo between core matrices adjacent in K given.
+__device__ __forceinline__ uint64_t make_desc_k(uint32_t saddr, uint32_t lbo, uint32_t sbo) {
+  return (uint64_t)((saddr >> 4) & 0x3FFFu) | (uint64_t)((lbo >> 4) & 0x3FFFu) << 16 |
+         (uint64_t)((sbo >> 4) & 0x3FFFu) << 32 | 1ull << 46;
+}
 // Instruction descriptor: D = f32, A/B = tf32 (2) or bf16 (1), both K-major, N, M.
 __host__ __device__ constexpr uint32_t make_idesc(int ab_fmt, int M, int N) {
   return (1u << 4) | ((uint32_t)ab_fmt << 7) | ((uint32_t)ab_fmt << 10) | ((uint32_t)(N >> 3) << 17) |
