@@ -140,7 +140,7 @@ struct DigitEntry {
 };
 
 struct DeviceCache {
-  std::map<std::tuple<int, int, int, int>, uint8_t*> shift;  // T^T of the sector-aligned stores
+  std::map<std::tuple<int, int, int, int>, uint8_t*> second;  // second operand images (second_table)
   unsigned* err = nullptr;
   int num_sms = 0;
   std::map<std::tuple<int, int, int>, double*> fp64;    // (form, degree, cell)
@@ -268,21 +268,24 @@ int tc_table(DeviceCache& c, int form, int degree, int cell, int prec, TcTable* 
   return COFFEE_OK;
 }
 
-int shift_table(DeviceCache& c, int form, int degree, int cell, int prec, const uint8_t** image) {
+// A second operand image of T for one (form, degree, cell, precision): the sector-aligned stores' on simplices, the
+// two-step sums' on prisms.
+int second_table(DeviceCache& c, int form, int degree, int cell, int prec, const uint8_t** image) {
   auto key = std::make_tuple(form, degree, cell, prec);
-  auto it = c.shift.find(key);
-  if (it == c.shift.end()) {
+  auto it = c.second.find(key);
+  if (it == c.second.end()) {
     std::vector<uint8_t> img;
-    build_shift_image(form, degree, cell, prec, img);
+    if (cell == CELL_PRISM) build_prism_sum_image(form, degree, img);
+    else build_shift_image(form, degree, cell, prec, img);
     uint8_t* d = nullptr;
     cudaError_t e = cudaMalloc(&d, img.size());
-    if (e != cudaSuccess) return cuda_fail(e, "cudaMalloc(shifted table)");
+    if (e != cudaSuccess) return cuda_fail(e, "cudaMalloc(second table)");
     e = cudaMemcpy(d, img.data(), img.size(), cudaMemcpyHostToDevice);
     if (e != cudaSuccess) {
       cudaFree(d);
-      return cuda_fail(e, "cudaMemcpy(shifted table)");
+      return cuda_fail(e, "cudaMemcpy(second table)");
     }
-    it = c.shift.emplace(key, d).first;
+    it = c.second.emplace(key, d).first;
   }
   *image = it->second;
   return COFFEE_OK;
@@ -338,8 +341,11 @@ int assemble_impl(const coffee_assemble_args* a, const uint32_t* map, int64_t nn
   if (a->cell == CELL_PRISM && a->precision != PREC_FP64) {
     if (!prism_tc_supported(a->form, a->degree, a->precision))
       return fail(COFFEE_ERR_UNSUPPORTED, "tensor-core prisms: MASS, HELMHOLTZ and ADVDIFF, P1-P4");
+    const bool sums = !map && prism_sum_tc_use(a->form);
     TcTable meta{};
-    if ((rc = tc_table(*c, a->form, a->degree, a->cell, a->precision, &meta)) != COFFEE_OK) return rc;
+    if (sums) rc = second_table(*c, a->form, a->degree, a->cell, PREC_TF32X3, &meta.image);
+    else rc = tc_table(*c, a->form, a->degree, a->cell, a->precision, &meta);
+    if (rc != COFFEE_OK) return rc;
     TcParams p{};
     p.coords = a->coords;
     p.c2v = a->cell2vert;
@@ -356,6 +362,11 @@ int assemble_impl(const coffee_assemble_args* a, const uint32_t* map, int64_t nn
     p.validate = validate ? 1 : 0;
     p.map = map;
     p.nnz = nnz;
+    if (sums) {
+      cudaError_t e = (cudaError_t)launch_prism_sum_tc(a->form, a->degree, p, c->num_sms, stream);
+      if (e != cudaSuccess) return cuda_fail(e, "launch(assemble_prism_sum_tc)");
+      return COFFEE_OK;
+    }
     std::string why;
     cudaError_t e = (cudaError_t)launch_prism_tc(a->form, a->degree, p, c->num_sms, stream, why);
     if (e != cudaSuccess) return cuda_fail(e, ("launch(assemble_prism_tc) " + why).c_str());
@@ -475,7 +486,7 @@ int assemble_impl(const coffee_assemble_args* a, const uint32_t* map, int64_t nn
     return COFFEE_OK;
   }
   if (!map && tc_shift_use(a->form, a->degree, a->cell, a->precision, p.ostride, p.tune, a->ncells) &&
-      (rc = shift_table(*c, a->form, a->degree, a->cell, a->precision, &p.shift_image)) != COFFEE_OK)
+      (rc = second_table(*c, a->form, a->degree, a->cell, a->precision, &p.shift_image)) != COFFEE_OK)
     return rc;
   cudaError_t e = map ? (cudaError_t)launch_tc_csr(a->form, a->cell, p, c->num_sms, stream, why)
                       : (cudaError_t)launch_tc(a->form, a->cell, p, c->num_sms, stream, why);

@@ -52,6 +52,9 @@ void prism_tensor(int form, int k, std::vector<double>& T, std::vector<double>& 
 void prism_rule_points(int n, std::vector<double>& pts, std::vector<double>& wts);
 int prism_points(int form, int k);
 void prism_sum_table(int form, int k, std::vector<double>& tab);
+void prism_factor_tables(int form, int k, std::vector<double>& pts, std::vector<double>& wts, std::vector<double>& psi,
+                         std::vector<double>& dpsi, std::vector<double>& zp, std::vector<double>& zw,
+                         std::vector<double>& zeta);
 
 // ---- error reporting (api.cu) ----
 int fail(int status, const std::string& msg);
@@ -284,6 +287,10 @@ int launch_csr_map(const int32_t* l2g, int64_t ncells, int nloc, const int64_t* 
 int tc_csr_supported(int form, int degree, int cell, int precision);
 void build_prism_tc_image(int form, int degree, int prec, std::vector<uint8_t>& img, TcTable& meta);
 int launch_prism_tc(int form, int degree, const TcParams& p, int num_sms, void* stream, std::string& why);
+// the same forms with the quadrature summed in two steps (k_prism_sum_tc.cu): local assembly
+bool prism_sum_tc_use(int form);
+void build_prism_sum_image(int form, int degree, std::vector<uint8_t>& img);
+int launch_prism_sum_tc(int form, int degree, const TcParams& p, int num_sms, void* stream);
 int launch_tc_csr(int form, int cell, const TcParams& p, int num_sms, void* stream, std::string& why);
 
 // Build the operand image on the host

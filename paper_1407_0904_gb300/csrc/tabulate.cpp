@@ -361,6 +361,30 @@ void prism_tensor(int form, int k, std::vector<double>& T, std::vector<double>& 
 // planar faces).
 int prism_points(int form, int k) { return burgers_like(form) ? (3 * k + 3) / 2 : k + 2; }
 
+// The factors of a prism's rule and basis: triangle points [p^2][2] and weights, psi [p^2][nt], its derivatives
+// [p^2][nt][2]; z's points and weights [p], zeta and zeta' [p][k+1][2].
+void prism_factor_tables(int form, int k, std::vector<double>& pts, std::vector<double>& wts, std::vector<double>& psi,
+                         std::vector<double>& dpsi, std::vector<double>& zp, std::vector<double>& zw,
+                         std::vector<double>& zeta) {
+  const int p = prism_points(form, k), nt = (k + 1) * (k + 2) / 2;
+  gauss_jacobi01(p, 0, zp, zw);
+  pts.clear();
+  wts.clear();
+  for (int i = 0; i < p; ++i)
+    for (int j = 0; j < p; ++j) {
+      pts.push_back(zp[i]);
+      pts.push_back(zp[j] * (1.0 - zp[i]));
+      wts.push_back(zw[i] * zw[j] * (1.0 - zp[i]));
+    }
+  psi.assign((size_t)p * p * nt, 0.0);
+  dpsi.assign((size_t)p * p * nt * 2, 0.0);
+  lagrange_basis(0, k, p * p, pts.data(), psi.data(), dpsi.data());
+  zeta.assign((size_t)p * (k + 1) * 2, 0.0);
+  for (int q = 0; q < p; ++q)
+    for (int c = 0; c <= k; ++c)
+      interval_basis(k, c, zp[q], zeta[((size_t)q * (k + 1) + c) * 2], zeta[((size_t)q * (k + 1) + c) * 2 + 1]);
+}
+
 // Tables of the direction-by-direction sums over a prism's points (p per direction; qt over the triangle's
 // p^2, qz over z's p), nt triangle and k+1 interval functions, pairs (i <= j) numbered j (j+1)/2 + i:
 //   [qt][nt][3]      psi, d_s psi, d_t psi
@@ -371,21 +395,11 @@ int prism_points(int form, int k) { return burgers_like(form) ? (3 * k + 3) / 2 
 //   [qt][3], [qz][2] points and weights (s, t, weight), (z, weight)
 void prism_sum_table(int form, int k, std::vector<double>& tab) {
   const int p = prism_points(form, k), nt = (k + 1) * (k + 2) / 2;
-  std::vector<double> g, w;
-  gauss_jacobi01(p, 0, g, w);
-  std::vector<double> psi((size_t)p * p * nt), dpsi((size_t)p * p * nt * 2), zeta((size_t)p * (k + 1) * 2);
+  std::vector<double> pts, wts, psi, dpsi, g, w, zeta;
+  prism_factor_tables(form, k, pts, wts, psi, dpsi, g, w, zeta);
   tab.clear();
-  for (int i = 0; i < p; ++i)
-    for (int j = 0; j < p; ++j) {
-      const int qt = i * p + j;
-      const double x[2] = {g[i], g[j] * (1.0 - g[i])};
-      lagrange_basis(0, k, 1, x, &psi[(size_t)qt * nt], &dpsi[(size_t)qt * nt * 2]);
-      for (int t = 0; t < nt; ++t) {
-        tab.push_back(psi[(size_t)qt * nt + t]);
-        tab.push_back(dpsi[((size_t)qt * nt + t) * 2]);
-        tab.push_back(dpsi[((size_t)qt * nt + t) * 2 + 1]);
-      }
-    }
+  for (size_t i = 0; i < psi.size(); ++i)
+    for (double v : {psi[i], dpsi[i * 2], dpsi[i * 2 + 1]}) tab.push_back(v);
   for (int qt = 0; qt < p * p; ++qt)
     for (int kind = 0; kind < 8; ++kind)
       for (int j = 0; j < nt; ++j)
@@ -397,18 +411,14 @@ void prism_sum_table(int form, int k, std::vector<double>& tab) {
           tab.push_back(v[kind]);
         }
   for (int q = 0; q < p; ++q)
-    for (int c = 0; c <= k; ++c)
-      interval_basis(k, c, g[q], zeta[((size_t)q * (k + 1) + c) * 2], zeta[((size_t)q * (k + 1) + c) * 2 + 1]);
-  for (int q = 0; q < p; ++q)
     for (int j = 0; j <= k; ++j)
       for (int i = 0; i <= j; ++i) {
         const double *a = &zeta[((size_t)q * (k + 1) + i) * 2], *b = &zeta[((size_t)q * (k + 1) + j) * 2];
         for (double v : {a[0] * b[0], a[0] * b[1], b[0] * a[1], a[1] * b[1]}) tab.push_back(v);
       }
   tab.insert(tab.end(), zeta.begin(), zeta.end());
-  for (int i = 0; i < p; ++i)
-    for (int j = 0; j < p; ++j)
-      for (double v : {g[i], g[j] * (1.0 - g[i]), w[i] * w[j] * (1.0 - g[i])}) tab.push_back(v);
+  for (int qt = 0; qt < p * p; ++qt)
+    for (double v : {pts[qt * 2], pts[qt * 2 + 1], wts[qt]}) tab.push_back(v);
   for (int q = 0; q < p; ++q)
     for (double v : {g[q], w[q]}) tab.push_back(v);
 }
