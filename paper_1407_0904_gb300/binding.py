@@ -6,6 +6,7 @@ through the C ABI declared in include/coffee.h, and turns status codes into
 exceptions. There is no CPU fallback: if the library is missing the calls raise.
 """
 import ctypes
+import functools
 import os
 
 import numpy as np
@@ -93,10 +94,14 @@ def dim(cell):
     return 2 if cell == TRIANGLE else 3
 
 
+_VERTS = {TRIANGLE: 3, TETRAHEDRON: 4, PRISM: 6}
+
+
 def verts_per_cell(cell):
-    return {TRIANGLE: 3, TETRAHEDRON: 4, PRISM: 6}[cell]
+    return _VERTS[cell]
 
 
+@functools.lru_cache(maxsize=256, typed=True)
 def ndof(form, degree, cell):
     n = lib().coffee_ndof(form, degree, cell)
     if n < 0:
@@ -195,9 +200,14 @@ def _ptr(t):
     return None if t is None else ctypes.c_void_p(t.data_ptr())
 
 
+def _address(t):
+    return None if t is None else t.data_ptr()
+
+
 def _stream_handle(stream):
-    s = torch.cuda.current_stream() if stream is None else stream
-    return ctypes.c_void_p(s.cuda_stream)
+    if stream is None:  # the current device's current stream, without a Stream object made for each call
+        return ctypes.c_void_p(torch._C._cuda_getCurrentRawStream(torch.cuda.current_device()))
+    return ctypes.c_void_p(stream.cuda_stream)
 
 
 def coef_width(form, degree, cell):
@@ -215,9 +225,10 @@ def check_shapes(form, degree, cell, coords, cell2vert, coef=None, cell2dof=None
     pointer is passed: the library receives bare pointers and cannot check extents."""
     d = dim(cell)
     nv = verts_per_cell(cell)
-    if cell2vert.dim() != 2 or cell2vert.shape[1] != nv:
+    sv, sx = cell2vert.shape, coords.shape
+    if len(sv) != 2 or sv[1] != nv:
         raise ValueError("cell2vert must be [ncells, %d]" % nv)
-    if coords.dim() != 2 or coords.shape[1] != d:
+    if len(sx) != 2 or sx[1] != d:
         raise ValueError("coords must be [nverts, %d]" % d)
     w = coef_width(form, degree, cell)
     if w == 0:
@@ -290,6 +301,7 @@ def make_args(form, degree, cell, coords, cell2vert, coef=None, cell2dof=None, p
     n = ndof(form, degree, cell)
     odt = torch.float64 if precision == FP64 else torch.float32
     shape = (ncells, n) if form == BURGERS_RESIDUAL else (ncells, n, n)  # element vectors or matrices
+    entries = n if form == BURGERS_RESIDUAL else n * n
     if out_stride:
         # padded rows: out is the flat buffer [ncells, out_stride] (see assemble)
         if out is None:
@@ -297,36 +309,30 @@ def make_args(form, degree, cell, coords, cell2vert, coef=None, cell2dof=None, p
                 out = torch.empty((ncells, out_stride), dtype=odt, device=coords.device)
         else:
             _dev(out, odt, "out")
-            if ncells and out.numel() < (ncells - 1) * out_stride + int(np.prod(shape[1:])):
-                raise ValueError("out must hold (ncells - 1) * out_stride + %d elements" % int(np.prod(shape[1:])))
+            if ncells and out.numel() < (ncells - 1) * out_stride + entries:
+                raise ValueError("out must hold (ncells - 1) * out_stride + %d elements" % entries)
     elif out is None:
         if alloc_out:
             out = torch.empty(shape, dtype=odt, device=coords.device)
     else:
         _dev(out, odt, "out")
-        if out.numel() != int(np.prod(shape)):
+        if out.numel() != ncells * entries:
             raise ValueError("out must hold %s elements" % "x".join(map(str, shape)))
     if ncoefnodes is None and coef is not None:
         ncoefnodes = coef.numel() // (1 + d) if form == ADVDIFF else coef.numel() // d
-    a = AssembleArgs()
-    a.form, a.degree, a.cell, a.precision, a.nu = form, degree, cell, precision, nu
-    a.coords, a.nverts = _ptr(coords), coords.shape[0]
-    a.cell2vert = _ptr(cell2vert)
-    a.coef, a.ncoefnodes = _ptr(coef), int(ncoefnodes or 0)
-    a.cell2dof = _ptr(cell2dof)
-    a.out, a.ncells = _ptr(out), ncells
-    a.flags = (FLAG_VALIDATE if validate else 0) | int(tune)
     if coords_split is not None:
         _dev(coords_split, torch.float32, "coords_split")
         if coords_split.numel() != 2 * coords.numel():
             raise ValueError("coords_split must hold 2 floats per coordinate (split_coords)")
-    a.coords_split = _ptr(coords_split)
     if coef_f32 is not None:
         _dev(coef_f32, torch.float32, "coef_f32")
         if coef is None or coef_f32.numel() != coef.numel():
             raise ValueError("coef_f32 must hold one float per coefficient of coef (round_coef)")
-    a.coef_f32 = _ptr(coef_f32)
-    a.out_stride = int(out_stride or 0)
+    # the fields in the structure's order, addresses as integers, in one call instead of seventeen assignments
+    a = AssembleArgs(form, degree, cell, precision, nu, _address(coords), coords.shape[0], _address(cell2vert),
+                     _address(coef), int(ncoefnodes or 0), _address(cell2dof), _address(out), ncells,
+                     (FLAG_VALIDATE if validate else 0) | int(tune), _address(coords_split), _address(coef_f32),
+                     int(out_stride or 0))
     return a, out
 
 
@@ -364,8 +370,8 @@ def _tuned_flags(form, degree, cell, precision):
     global _tune_cache
     if precision == FP64 or form in (BURGERS_JAC, BURGERS_RESIDUAL):
         return 0
-    from . import tune as _tune
     if _tune_cache is None:
+        from . import tune as _tune
         try:
             _tune_cache = _tune.load_cache()
         except (OSError, ValueError):
@@ -373,6 +379,12 @@ def _tuned_flags(form, degree, cell, precision):
     ent = _tune_cache.get("%d/%d/%d/%d" % (form, degree, cell, precision))
     if ent is not None:
         return int(ent.get("flags", 0))
+    return _model_flags(form, degree, cell, precision)
+
+
+@functools.lru_cache(maxsize=256, typed=True)
+def _model_flags(form, degree, cell, precision):
+    from . import tune as _tune
     return _tune.model_flags(ndof(form, degree, cell) ** 2,
                              assemble_path(form, degree, cell, precision, FLAG_CUDA_CORES) == 2)
 
