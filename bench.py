@@ -243,7 +243,7 @@ def prism_fma(form, k):
     if form == BURGERS_RESIDUAL:
         return point + p ** 3 * nz * 12 + p * p * nt * nz * 9
     ntp, nzp = nt * (nt + 1) // 2, nz * (nz + 1) // 2
-    fields, per = {MASS: (1, 1), HELMHOLTZ: (9, 13), ADVDIFF: (12, 18), BURGERS_JAC: (21, 27)}[form]
+    fields, per = {MASS: (1, 1), HELMHOLTZ: (9, 8), ADVDIFF: (12, 11), BURGERS_JAC: (21, 20)}[form]
     return point + p ** 3 * nzp * fields + p * p * ntp * nzp * per
 
 

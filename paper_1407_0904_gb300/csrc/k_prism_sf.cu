@@ -11,18 +11,19 @@
 //   beta_a = w|det| (K b)_a,   A_ij = sum_q M phi_i phi_j + V_ab d_a phi_i d_b phi_j + phi_i beta_a d_a phi_j:
 // first, per triangle point and pair (iz <= jz), the factors are summed over qz against the products of
 // zeta and zeta' (8 to 21 fields); then, per pair (it <= jt), over qt against the products of psi and its
-// derivatives. One such quadruple gives the up to four entries that exchange it with jt and iz with jz: M and
-// the V_ss, V_st, V_tt, V_zz terms are common to them, the V_sz, V_tz terms take two values, the beta terms
-// two for the exchange of it and jt plus two for that of iz and jz.
+// derivatives. One such quadruple gives the up to four entries that exchange it with jt and iz with jz, which
+// differ only in signs once the products of psi and d psi are taken as half sums and differences (below).
 //
 // The FP64 pipe (2 FMAs per cycle and SM) bounds this as it did the sums over all points that stood here
 // before (Burgers Jacobian P2: 435,000 FMAs a cell, 33.7 ms for 27,648 cells; Helmholtz P2 145,000). The two
-// steps take 27 FMAs per quadruple and triangle point (Burgers; Helmholtz 13), 54,000 in all for P2 where
-// the direct sum takes 21 per entry and point. u and its derivatives at the points are formed the same way.
-// Measured, now / the direct sums: Burgers Jacobian 27,648 P2 3.77 / 33.65 ms (54,000 + 9,000 FMAs, 0.78 of the FP64
-// rate), 2000 P4 9.7 / 279 ms; its residual P2 0.96 / 2.83 ms; 27,648 P2 Helmholtz 1.74 / 7.62, advection-
-// diffusion 2.40 / 9.81, mass 0.32 / 1.24 ms; 60,000 P1 Helmholtz 0.62 / 1.74 ms. 300 cells: P1 28-42 us as
-// launched from Python against 33-81, P4 0.05-1.4 ms against 1.1-70.
+// steps take 20 FMAs per quadruple and triangle point (Burgers; Helmholtz 8, advection-diffusion 11; with the
+// exchanged entries summed one by one 27, 13, 18), 40,000 in all for P2 where the direct sum takes 21 per entry and
+// point. u and its derivatives at the points are formed the same way.
+// Measured, now / the exchanged entries one by one / the direct sums: Burgers Jacobian 27,648 P2 3.18 / 3.77 /
+// 33.65 ms (40,000 + 9,000 FMAs, 0.79 of the FP64 rate), 2000 P4 7.5 / 9.7 / 279 ms; 27,648 P2 Helmholtz 1.30 / 1.74 /
+// 7.62, advection-diffusion 1.80 / 2.40 / 9.81 ms. Now / the direct sums: residual P2 0.96 / 2.83, mass 0.32 / 1.24 ms;
+// 60,000 P1 Helmholtz 0.58 / 1.74 ms; 300 cells P1 16-36 us as launched from Python against 33-81, P4 0.05-1.1 ms
+// against 1.1-70.
 // A block holds one cell (P1: seven, residual P2: two), its factors and fields in shared memory, and several
 // blocks share an SM, so that one's table reads and barriers hide behind another's FMAs.
 #include <cuda_runtime.h>
@@ -42,7 +43,8 @@ struct Sf {
   static constexpr int NM = FORM == FORM_BURGERS ? 9 : FORM == FORM_ADVDIFF ? 0 : 1;  // M fields
   static constexpr bool V = FORM != FORM_MASS, BETA = FORM == FORM_ADVDIFF || FORM == FORM_BURGERS;
   static constexpr int NF = res ? 12 : NM + (V ? 6 : 0) + (BETA ? 3 : 0);              // factors of a point
-  static constexpr int NFLD = res ? 9 : NM + (V ? 8 : 0) + (BETA ? 4 : 0);             // fields of (qt, z pair)
+  static constexpr int NB = NM == 9 ? 9 : 0;                                           // of them, a block's own (M)
+  static constexpr int NFLD = res ? 9 : !V ? 1 : BETA ? NB + 11 : 8;                   // fields of (qt, z pair)
   static constexpr int items = res ? 3 * n : NTP * NZP;                                // of one cell, last step
   static constexpr int CELLS = DEG == 1 ? 7 : res && DEG == 2 ? 2 : 1;
   static constexpr int THREADS = DEG == 3 && !res ? 192 : DEG == 4 && !res ? 320 : 128;
@@ -87,7 +89,7 @@ template <int FORM, int DEG, bool CSR>
 __global__ void __launch_bounds__(Sf<FORM, DEG>::THREADS) k_prism_sf(const PrismParams p) {
   using S = Sf<FORM, DEG>;
   constexpr int QT = S::QT, QZ = S::QZ, Q = S::Q, NT = S::NT, NZ = S::NZ, n = S::n, N = S::N, NF = S::NF, NFLD = S::NFLD,
-                NTP = S::NTP, NZP = S::NZP, NM = S::NM, CELLS = S::CELLS, THREADS = S::THREADS;
+                NTP = S::NTP, NZP = S::NZP, NM = S::NM, NB = S::NB, CELLS = S::CELLS, THREADS = S::THREADS;
   extern __shared__ double sm[];
   double* sF = sm;                                  // [CELLS][Q][NF]
   double* sS = sF + CELLS * Q * NF;                 // [CELLS][QT][NZP or NZ][NFLD]
@@ -228,70 +230,93 @@ __global__ void __launch_bounds__(Sf<FORM, DEG>::THREADS) k_prism_sf(const Prism
     }
     __syncthreads();
     if constexpr (!S::res) {
-      // ---- sums over z: fields M.., V_ss, V_st, V_tt (zeta_i zeta_j), V_zz (zeta'_i zeta'_j), V_sz and V_tz with
-      // zeta_i zeta'_j and with zeta_j zeta'_i, beta_s, beta_t (zeta_i zeta_j), beta_z with the two mixed ones ----
+      // ---- sums over z of M zeta_i zeta_j, V_ss, V_st, V_tt (zeta_i zeta_j), V_zz (zeta'_i zeta'_j), V_sz and V_tz
+      // with zeta_i zeta'_j (1) and with zeta_j zeta'_i (2), beta_s, beta_t (zeta_i zeta_j), beta_z (1, 2); of these
+      // the fields, in the order of the tables they meet below ----
       for (int i = tid; i < nc * QT * NZP; i += THREADS) {
         const int zp = i % NZP, qt = i / NZP % QT, c = i / (NZP * QT);
-        double a[NFLD];
+        double m[NM > 0 ? NM : 1], ss = 0.0, st = 0.0, tt = 0.0, zz = 0.0, sz1 = 0.0, sz2 = 0.0, tz1 = 0.0, tz2 = 0.0,
+               bs = 0.0, bt = 0.0, bz1 = 0.0, bz2 = 0.0;
 #pragma unroll
-        for (int k = 0; k < NFLD; ++k) a[k] = 0.0;
+        for (int k = 0; k < (NM > 0 ? NM : 1); ++k) m[k] = 0.0;
         const double* f = sF + (size_t)(c * Q + qt * QZ) * NF;
 #pragma unroll 2
         for (int qz = 0; qz < QZ; ++qz, f += NF) {
           const double* w = sZ + (qz * NZP + zp) * 4;
           const double w0 = w[0], w1 = w[1], w2 = w[2], w3 = w[3];
 #pragma unroll
-          for (int k = 0; k < NM; ++k) a[k] = fma(f[k], w0, a[k]);
+          for (int k = 0; k < NM; ++k) m[k] = fma(f[k], w0, m[k]);
           if constexpr (S::V) {  // pairs ss, st, sz, tt, tz, zz
-            a[NM] = fma(f[NM], w0, a[NM]);
-            a[NM + 1] = fma(f[NM + 1], w0, a[NM + 1]);
-            a[NM + 2] = fma(f[NM + 3], w0, a[NM + 2]);
-            a[NM + 3] = fma(f[NM + 5], w3, a[NM + 3]);
-            a[NM + 4] = fma(f[NM + 2], w1, a[NM + 4]);
-            a[NM + 5] = fma(f[NM + 2], w2, a[NM + 5]);
-            a[NM + 6] = fma(f[NM + 4], w1, a[NM + 6]);
-            a[NM + 7] = fma(f[NM + 4], w2, a[NM + 7]);
+            ss = fma(f[NM], w0, ss);
+            st = fma(f[NM + 1], w0, st);
+            tt = fma(f[NM + 3], w0, tt);
+            zz = fma(f[NM + 5], w3, zz);
+            sz1 = fma(f[NM + 2], w1, sz1);
+            sz2 = fma(f[NM + 2], w2, sz2);
+            tz1 = fma(f[NM + 4], w1, tz1);
+            tz2 = fma(f[NM + 4], w2, tz2);
           }
           if constexpr (S::BETA) {
-            a[NM + 8] = fma(f[NM + 6], w0, a[NM + 8]);
-            a[NM + 9] = fma(f[NM + 7], w0, a[NM + 9]);
-            a[NM + 10] = fma(f[NM + 8], w1, a[NM + 10]);
-            a[NM + 11] = fma(f[NM + 8], w2, a[NM + 11]);
+            bs = fma(f[NM + 6], w0, bs);
+            bt = fma(f[NM + 7], w0, bt);
+            bz1 = fma(f[NM + 8], w1, bz1);
+            bz2 = fma(f[NM + 8], w2, bz2);
           }
         }
         double* o = sS + c * S::S1 + (qt * NZP + zp) * NFLD;
+        if constexpr (!S::V) {
+          o[0] = m[0];
+        } else {
 #pragma unroll
-        for (int k = 0; k < NFLD; ++k) o[k] = a[k];
+          for (int k = 0; k < NB; ++k) o[k] = m[k];
+          o += NB;
+          o[0] = ss, o[1] = st, o[2] = tt;
+          o[3] = (sz1 + sz2) + bs, o[4] = (tz1 + tz2) + bt;
+          o[5] = (sz1 - sz2) - bs, o[6] = (tz1 - tz2) - bt;
+          if constexpr (S::BETA) {
+            o[7] = (sz1 - sz2) + bs, o[8] = (tz1 - tz2) + bt;
+            o[9] = zz + bz1, o[10] = zz + bz2;
+          } else {
+            o[7] = zz + m[0];
+          }
+        }
       }
       __syncthreads();
-      // ---- sums over the triangle's points, one quadruple (it <= jt, iz <= jz) per thread ----
+      // ---- sums over the triangle's points, one quadruple (it <= jt, iz <= jz) per thread. Exchanging it with jt
+      // leaves P+, R+ = (d psi_it psi_jt + psi_it d psi_jt) / 2 as they are and turns the sign of P-, R-; exchanging
+      // iz with jz turns that of V_sz, V_tz (1) - (2). So with x the beta_s field the four entries are
+      //   C +- sum (sz1 - sz2 - x) P- + .. + sum (zz + bz1) T    and    C -+ sum (sz1 - sz2 + x) P- + .. + sum (zz + bz2) T,
+      // C the sum of the ss, st, tt terms and of (sz1 + sz2 + x) P+ + (tz1 + tz2 + y) R+, common to all. ----
       for (int i = tid; i < nc * S::items; i += THREADS) {
         const int c = i / S::items, k = i % S::items, zp = k / NTP, tq = k % NTP;
-        double M[NM > 0 ? NM : 1], s1 = 0.0, E1 = 0.0, E2 = 0.0, u1 = 0.0, u2 = 0.0, v1 = 0.0, v2 = 0.0;
+        double M[NB > 0 ? NB : 1], C = 0.0, G1 = 0.0, G2 = 0.0, v1 = 0.0, v2 = 0.0;
 #pragma unroll
-        for (int x = 0; x < (NM > 0 ? NM : 1); ++x) M[x] = 0.0;
+        for (int x = 0; x < (NB > 0 ? NB : 1); ++x) M[x] = 0.0;
         const double* f = sS + c * S::S1 + zp * NFLD;
         const double* tt = tp + tq;
 #pragma unroll 2
         for (int qt = 0; qt < QT; ++qt, f += NZP * NFLD, tt += 8 * NTP) {
           const double T = __ldg(tt);
 #pragma unroll
-          for (int x = 0; x < NM; ++x) M[x] = fma(f[x], T, M[x]);
+          for (int x = 0; x < NB; ++x) M[x] = fma(f[x], T, M[x]);
           if constexpr (S::V) {
-            const double Tss = __ldg(tt + NTP), Tst = __ldg(tt + 2 * NTP), Ttt = __ldg(tt + 3 * NTP);
-            const double Pij = __ldg(tt + 4 * NTP), Pji = __ldg(tt + 5 * NTP), Rij = __ldg(tt + 6 * NTP),
-                         Rji = __ldg(tt + 7 * NTP);  // d_s psi_it psi_jt and exchanged, d_t ..
-            s1 = fma(f[NM], Tss, fma(f[NM + 1], Tst, fma(f[NM + 2], Ttt, fma(f[NM + 3], T, s1))));
-            E1 = fma(f[NM + 4], Pij, fma(f[NM + 5], Pji, fma(f[NM + 6], Rij, fma(f[NM + 7], Rji, E1))));
-            E2 = fma(f[NM + 4], Pji, fma(f[NM + 5], Pij, fma(f[NM + 6], Rji, fma(f[NM + 7], Rij, E2))));
+            const double* h = f + NB;
+            const double Pp = __ldg(tt + 4 * NTP), Pm = __ldg(tt + 5 * NTP), Rp = __ldg(tt + 6 * NTP), Rm = __ldg(tt + 7 * NTP);
+            C = fma(h[0], __ldg(tt + NTP), fma(h[1], __ldg(tt + 2 * NTP), fma(h[2], __ldg(tt + 3 * NTP), C)));
+            C = fma(h[3], Pp, fma(h[4], Rp, C));
+            G1 = fma(h[5], Pm, fma(h[6], Rm, G1));
             if constexpr (S::BETA) {
-              u1 = fma(f[NM + 8], Pji, fma(f[NM + 9], Rji, u1));
-              u2 = fma(f[NM + 8], Pij, fma(f[NM + 9], Rij, u2));
-              v1 = fma(f[NM + 10], T, v1);
-              v2 = fma(f[NM + 11], T, v2);
+              G2 = fma(h[7], Pm, fma(h[8], Rm, G2));
+              v1 = fma(h[9], T, v1);
+              v2 = fma(h[10], T, v2);
+            } else {
+              C = fma(h[7], T, C);
             }
+          } else {
+            C = fma(f[0], T, C);
           }
         }
+        if constexpr (!S::BETA) G2 = G1;
         if (sbad[c]) continue;
         int jt = 0, jz = 0;  // tq = jt (jt + 1) / 2 + it, zp = jz (jz + 1) / 2 + iz
         while ((jt + 1) * (jt + 2) / 2 <= tq) ++jt;
@@ -305,7 +330,7 @@ __global__ void __launch_bounds__(Sf<FORM, DEG>::THREADS) k_prism_sf(const Prism
             for (int cj = 0; cj < (S::burgers ? 3 : 1); ++cj) {
               const int at = (ci * n + row) * N + cj * n + col;
               double v = ci == cj ? d : 0.0;
-              if constexpr (NM > 0) v += M[NM == 9 ? ci * 3 + cj : 0];
+              if constexpr (NB > 0) v += M[ci * 3 + cj];
               if constexpr (CSR) {
                 const uint32_t pos = __ldg(p.map + csr_map_index(e, at, (N * N + 3) & ~3));
                 if (pos < (uint64_t)p.nnz) atomicAdd(static_cast<double*>(p.out) + pos, v);
@@ -315,10 +340,10 @@ __global__ void __launch_bounds__(Sf<FORM, DEG>::THREADS) k_prism_sf(const Prism
               }
             }
         };
-        put(iz * NT + it, jz * NT + jt, s1 + E1 + u1 + v1);
-        if (it != jt) put(iz * NT + jt, jz * NT + it, s1 + E2 + u2 + v1);
-        if (iz != jz) put(jz * NT + it, iz * NT + jt, s1 + E2 + u1 + v2);
-        if (it != jt && iz != jz) put(jz * NT + jt, iz * NT + it, s1 + E1 + u2 + v2);
+        put(iz * NT + it, jz * NT + jt, C + G1 + v1);
+        if (it != jt) put(iz * NT + jt, jz * NT + it, C - G1 + v1);
+        if (iz != jz) put(jz * NT + it, iz * NT + jt, C - G2 + v2);
+        if (it != jt && iz != jz) put(jz * NT + jt, iz * NT + it, C + G2 + v2);
       }
     } else {
       // ---- residual: sums over z of a_c zeta + gamma_cz zeta', gamma_cs zeta, gamma_ct zeta, then over qt ----

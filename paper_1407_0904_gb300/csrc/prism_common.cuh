@@ -5,9 +5,9 @@
 namespace coffee {
 namespace {
 
-// Factors of one quadrature point pq = (s, t, z, w) of a prism |det J| (1, (K K^T)_ab) or |det J| (eps (K K^T)_ab, (K b)_a): J from
-// the per-cell bilinear coefficients (d/ds = A + z B, d/dt = C + z D, d/dz = E + s F + t G), and
-// for advection-diffusion eps and b from the six vertex values CF. Every factor is linear in w.
+// Factors of one quadrature point pq = (s, t, z, w) of a prism, |det J| (1, (K K^T)_ab) or |det J| (eps (K K^T)_ab,
+// (K b)_a): J from the per-cell bilinear coefficients (d/ds = A + z B, d/dt = C + z D, d/dz = E + s F + t G), and for
+// advection-diffusion eps and b from the six vertex values CF. Every factor is linear in w.
 template <int KQ>
 __device__ __forceinline__ void prism_point_factors(const float4 pq, const float (&JA)[3], const float (&JB)[3],
                                                     const float (&JC)[3], const float (&JD)[3], const float (&JE)[3],
