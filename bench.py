@@ -589,15 +589,23 @@ def run_ours(args):
                     "peak_source": "FP64 FMA loop measured on this GPU (coffee_peak_fp64)", "flops_per_cell": flops,
                     "kernel_ms": launch_ms, "hbm_gbs": achieved}
         else:
-            # tensor pipe: executed MMA flops (K padded to the 64-byte chunk plus the centre
-            # chunk, outputs to 128-row slices, one pass per product of operand parts the
-            # precision keeps) against the tf32/bf16 dense peak
+            # tensor pipe: executed MMA flops, one pass per product of operand parts the kernel keeps, against the
+            # tf32/bf16 dense peak
             tf32 = prec in (coffee.TF32, coffee.TF32X3)
-            kc = 16 if tf32 else 32
-            kpad = -(-K // kc) * kc + kc
-            npad = -(-(ndof * ndof) // 128) * 128
-            passes = {coffee.TF32: 1, coffee.TF32X3: 3, coffee.BF16: 2, coffee.BF16X3: 6}[prec]
-            executed = 2.0 * kpad * npad * passes
+            if form in (HELMHOLTZ, ADVDIFF):
+                # summed over z first: 8 columns a triangle point and the centre's (two points a chunk), 128 rows a
+                # tile of a lane quadrant's cells times four, split tf32 whatever the precision
+                nt, nz, qt = (degree + 1) * (degree + 2) // 2, degree + 1, (degree + 2) ** 2
+                rows = nz * (nz + 1) // 2 if form == HELMHOLTZ else nz * nz
+                flops = 2.0 * 8 * qt * (rows * nt * nt + (degree + 2) * rows) + 250.0 * Q
+                tf32 = True
+                executed = 2.0 * 16 * (qt // 2 + 1) * -(-(nt * nt) // 16) * 16 * 3 * 32.0 / (32 // rows)
+            else:  # all points at once: K padded to the 64-byte chunk plus the centre chunk, outputs to 128-row slices
+                kc = 16 if tf32 else 32
+                kpad = -(-K // kc) * kc + kc
+                npad = -(-(ndof * ndof) // 128) * 128
+                passes = {coffee.TF32: 1, coffee.TF32X3: 3, coffee.BF16: 2, coffee.BF16X3: 6}[prec]
+                executed = 2.0 * kpad * npad * passes
             if tf32:
                 peak_t = device_peaks(coffee)["tf32_tflops"]
                 src = "tcgen05 kind::tf32 loop measured on this GPU (coffee_peak_mma, N=256)"
