@@ -15,9 +15,9 @@
 //
 // Every precision runs the split-tf32 operands: the MMAs do not bound it (one pass instead of three saved 5-15 %),
 // and factors summed before they are rounded average their rounding errors less than single points do.
-// Bound by shared memory: the MMAs' operands (78 of 7.5 KB a P3 tile), the fields' reads of the factors and the
-// chunks' stores take 0.9 of its cycles. Factors and fields are separate warps, two tiles of factors in flight,
-// because in the same warps one after the other they took 24,000 cycles a P3 tile for 16,800 now; matrix rows put
+// Bound by shared memory: the MMAs' operands (78 of 7.5 KB a P3 tile), the fields' reads of the factors, the
+// chunks' stores and the epilogue's staging. Factors and fields are separate warps, two tiles of factors in flight,
+// because in the same warps one after the other they took 24,000 cycles a P3 tile for 16,800; matrix rows put
 // together in shared memory because stores of a thread's own runs of nt entries touch 32 sectors each (P4: 48,000
 // cycles a tile of stores, 22,000 now).
 //
@@ -57,6 +57,11 @@ struct Zs {
   static constexpr int NT = (DEG + 1) * (DEG + 2) / 2, NZ = DEG + 1, n = NT * NZ;
   static constexpr int NR = sym ? NZ * (NZ + 1) / 2 : NZ * NZ;    // rows of a cell
   static constexpr int CPW = 32 / NR, CT = 4 * CPW;               // cells of a lane quadrant, of a tile
+  // Rows of one cell a field thread forms (z pairs j and j + HR): its factors are read once for both, 4,200 -> 2,100
+  // cycles of shared-memory reads a P3 tile (Helmholtz P3 262 -> 237 us, advection-diffusion P2 354 -> 316). Not P1,
+  // whose ten cells a quadrant would not fit sixteen threads, nor P4, which has two stages only (see ZLayout).
+  static constexpr int RPT = DEG == 2 || DEG == 3 ? 2 : 1, HR = (NR + RPT - 1) / RPT;
+  static_assert(RPT == 1 || CPW * HR <= 16, "sixteen threads a lane quadrant");
   static constexpr int NO = NT * NT, NP = (NO + 15) / 16 * 16;
   static constexpr int FS = sym ? 8 : 12;                         // floats of a point's factors in shared memory
   static constexpr int CS = Q * FS + (36 - Q * FS % 32) % 32;     // of a cell's: cells start 4 banks apart
@@ -78,7 +83,10 @@ struct ZLayout : Zs<FORM, DEG> {
   static constexpr int fit = (227 * 1024 - FIXED) / S::STAGE;
   static constexpr int NST = fit < Z_MAX_STAGES ? fit : Z_MAX_STAGES;
   static constexpr int SMEM = NST * S::STAGE + FIXED;
-  static_assert(NST >= 2, "two stages at least");
+  // RPT = 2: a thread waits for the slots of every other chunk, k' = k - 2 or, from one tile to the next, k - 3 before
+  // k. That chunk k' - NST was consumed tells it that chunk k - 2 NST was, and with it which of the slot's two phases the
+  // parity means, only if k - k' <= NST.
+  static_assert(NST >= (S::RPT == 2 ? 3 : 2), "stages");
 };
 
 __device__ __forceinline__ void tmem_ld1(uint32_t taddr, uint32_t* v) {
@@ -159,7 +167,7 @@ __global__ void __launch_bounds__(Z_THREADS, 1) k_prism_sum_tc(const TcParams p)
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < NST; ++s) {
-      mbar_init(smem_u32(&bars->full[s]), Z_NFIELD + 1);
+      mbar_init(smem_u32(&bars->full[s]), Z_NFIELD / S::RPT + 1);
       mbar_init(smem_u32(&bars->empty[s]), 1);
     }
     for (int r = 0; r < 2; ++r) {
@@ -224,25 +232,30 @@ __global__ void __launch_bounds__(Z_THREADS, 1) k_prism_sum_tc(const TcParams p)
       mbar_arrive(smem_u32(&bars->ffull[f]));
     }
   } else if (warp >= Z_FIELD0 && warp < MMA_WARP) {
-    // ---------------- fields: one (cell, z pair) per thread, half of a chunk's triangle points ----------------
-    const int id = threadIdx.x - Z_FIELD0 * 32, row = id & (BM - 1), sub = id >> 7;
-    const bool used = lane < CPW * NR;
-    const int cl = (row >> 5) * CPW + (used ? lane / NR : 0), zi = lane % NR;
-    float4 w[QZ];
+    // ---------------- fields: RPT (cell, z pair) rows per thread, one of a chunk's two triangle points ----------------
+    // RPT = 1: two chunks at once, 128 rows x 2 points; RPT = 2: each half of the warps every other chunk
+    constexpr int RPT = S::RPT, HR = S::HR, LANES = BM / RPT, UC = 3 - RPT;
+    const int id = threadIdx.x - Z_FIELD0 * 32, at = id % LANES, sub = id / LANES & 1, half = RPT == 2 ? id >> 7 : 0;
+    const int q = at / (32 / RPT), l = at % (32 / RPT), cw = l % CPW, j = l / CPW;
+    const bool used = j < HR;
+    const int cl = q * CPW + cw;
+    float4 w[RPT][QZ];
 #pragma unroll
-    for (int z = 0; z < QZ; ++z) w[z] = __ldg(ztab + z * NR + zi);
+    for (int y = 0; y < RPT; ++y)
+#pragma unroll
+      for (int z = 0; z < QZ; ++z) w[y][z] = __ldg(ztab + z * NR + (j + y * HR < NR ? j + y * HR : 0));
     uint32_t c = 0, i = 0;
     bool ok = true;
-    for (int64_t t = blockIdx.x; t < ntiles && ok; t += gridDim.x, ++i) {
+    for (int64_t t = blockIdx.x; t < ntiles && ok; t += gridDim.x, ++i, c += NKC) {
       const uint32_t f = i & 1u, r = i % Z_NREC;
       // the record: its words are written before the factors that ffull stands for
       if (!mbar_wait(smem_u32(&bars->cfull[r]), (i / Z_NREC) & 1u, p.err)) break;
       if (!mbar_wait(smem_u32(&bars->ffull[f]), (i >> 1) & 1u, p.err)) break;
       const float* F = sF + (f * CT + cl) * CS;
-      for (int kc = 0; kc < NKC && ok; kc += 2) {  // two chunks at once: two independent chains a thread
-        float x[2][8] = {};
+      for (int kc = half; kc < NKC && ok; kc += 2) {
+        float x[UC][RPT][8] = {};
 #pragma unroll
-        for (int u = 0; u < 2; ++u) {
+        for (int u = 0; u < UC; ++u) {
           const int qt = (kc + u) * Z_QC + sub;
           if (used && qt < QT) {
             const float4* f4 = reinterpret_cast<const float4*>(F + qt * QZ * FS);
@@ -251,23 +264,33 @@ __global__ void __launch_bounds__(Z_THREADS, 1) k_prism_sum_tc(const TcParams p)
               float g[FS];
 #pragma unroll
               for (int v = 0; v < FS / 4; ++v) *reinterpret_cast<float4*>(g + 4 * v) = f4[z * (FS / 4) + v];
-              add_fields<S::sym>(g, w[z], x[u]);
+#pragma unroll
+              for (int y = 0; y < RPT; ++y) add_fields<S::sym>(g, w[y][z], x[u][y]);
             }
           } else if (used && qt == QT) {
-            add_fields<S::sym>(sC + (r * CT + cl) * Z_REC + 45, __ldg(ztab + QZ * NR + zi), x[u]);
+#pragma unroll
+            for (int y = 0; y < RPT; ++y)
+              add_fields<S::sym>(sC + (r * CT + cl) * Z_REC + 45, __ldg(ztab + QZ * NR + (j + y * HR < NR ? j + y * HR : 0)), x[u][y]);
           }
         }
 #pragma unroll
-        for (int u = 0; u < 2; ++u) {
+        for (int u = 0; u < UC; ++u) {
           if (kc + u >= NKC) break;
-          const int s = (int)(c % NST);
-          if (!mbar_wait(empty + 8 * s, ((c / NST) & 1u) ^ 1u, p.err)) { ok = false; break; }
+          const uint32_t k = c + kc + u;
+          const int s = (int)(k % NST);
+          if (!mbar_wait(empty + 8 * s, ((k / NST) & 1u) ^ 1u, p.err)) { ok = false; break; }
           uint8_t* a = smem + (size_t)s * L::STAGE;
-          store_unit<true, Z_GP>(a + canon_off(row, sub * 32, Z_CB), BM * Z_CB, &x[u][0]);
-          store_unit<true, Z_GP>(a + canon_off(row, sub * 32 + 16, Z_CB), BM * Z_CB, &x[u][4]);
+#pragma unroll
+          for (int y = 0; y < RPT; ++y) {
+            // (the rows past the cells', which RPT = 2 leaves as they are, feed accumulator rows that nothing reads)
+            const int zi = j + y * HR, row = q * 32 + zi * CPW + cw;
+            if (RPT == 1 || (used && zi < NR)) {
+              store_unit<true, Z_GP>(a + canon_off(row, sub * 32, Z_CB), BM * Z_CB, &x[u][y][0]);
+              store_unit<true, Z_GP>(a + canon_off(row, sub * 32 + 16, Z_CB), BM * Z_CB, &x[u][y][4]);
+            }
+          }
           fence_proxy_async();
           mbar_arrive(full + 8 * s);
-          ++c;
         }
       }
       if (!ok) break;
@@ -398,7 +421,7 @@ __global__ void __launch_bounds__(Z_THREADS, 1) k_prism_sum_tc(const TcParams p)
   } else {
     // ---------------- epilogue ----------------
     constexpr int VEC = n % 4 == 0 ? 4 : n % 2 == 0 ? 2 : 1;
-    const int zi = lane % NR, cw = lane / NR;
+    const int zi = lane / CPW < NR ? lane / CPW : 0, cw = lane / CPW < NR ? lane % CPW : CPW;
     int iz = zi / NZ, jz = zi % NZ;
     if (S::sym) {
       for (jz = 0; (jz + 1) * (jz + 2) / 2 <= zi;) ++jz;
@@ -513,14 +536,14 @@ cudaError_t launch_zd(int degree, const TcParams& p, int num_sms, cudaStream_t s
 
 // All of both forms at any count. Graph-replayed times, us, split tf32, one contraction over all points | here:
 //   cells                 7           3000          P1 250,000, P2 110,592, P3 55,296, P4 16,000
-//   HELMHOLTZ   P1    25 | 11       27 | 13       280 | 147
-//               P2    53 | 13       56 | 14       297 | 196
-//               P3   441 | 18      436 | 26      1301 | 263
-//               P4  2269 | 28     2226 | 59      2231 | 226
+//   HELMHOLTZ   P1    25 | 10       27 | 13       280 | 148
+//               P2    53 | 13       56 | 14       297 | 188
+//               P3   441 | 17      436 | 25      1301 | 237
+//               P4  2269 | 26     2226 | 55      2231 | 207
 //   ADVDIFF     P1    36 | 12       37 | 12       412 | 237
-//               P2    75 | 15       77 | 21       417 | 354
-//               P3   643 | 18      626 | 33      1871 | 360
-//               P4  3306 | 26     3202 | 82      3210 | 390
+//               P2    75 | 14       77 | 20       417 | 316
+//               P3   643 | 17      626 | 32      1871 | 336
+//               P4  3306 | 25     3202 | 81      3210 | 381
 // The plain tf32 and bf16 operands of the other kernel: 267-391 us at P1, 258-387 at P2, 1104 and more above.
 // Its error against 64 bits is 1.7-4.8 times this one's in split tf32, 1.2-3.8 times in bf16x3.
 // MASS (K = (k+2)^3) and the CSR forms stay with the other.
