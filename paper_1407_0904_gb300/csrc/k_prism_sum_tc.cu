@@ -15,8 +15,8 @@
 //
 // Every precision runs the split-tf32 operands: the MMAs do not bound it (one pass instead of three saved 5-15 %),
 // and factors summed before they are rounded average their rounding errors less than single points do.
-// Bound by shared memory: the MMAs' operands (78 of 7.5 KB a P3 tile), the fields' reads of the factors, the
-// chunks' stores and the epilogue's staging. Factors and fields are separate warps, two tiles of factors in flight,
+// Bound by shared memory (L1 data pipe 72 % busy beside the MMAs' operands, 78 of 7.5 KB a P3 tile) and, with it, the
+// latency of the fields' and the epilogue's chains: a seventh fewer wavefronts by padding gained 2 % at P3, lost 3 % at P1. Factors and fields are separate warps, two tiles of factors in flight,
 // because in the same warps one after the other they took 24,000 cycles a P3 tile for 16,800; matrix rows put
 // together in shared memory because stores of a thread's own runs of nt entries touch 32 sectors each (P4: 48,000
 // cycles a tile of stores, 22,000 now).
