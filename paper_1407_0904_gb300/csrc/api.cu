@@ -341,7 +341,7 @@ int assemble_impl(const coffee_assemble_args* a, const uint32_t* map, int64_t nn
   if (a->cell == CELL_PRISM && a->precision != PREC_FP64) {
     if (!prism_tc_supported(a->form, a->degree, a->precision))
       return fail(COFFEE_ERR_UNSUPPORTED, "tensor-core prisms: MASS, HELMHOLTZ and ADVDIFF, P1-P4");
-    const bool sums = !map && prism_sum_tc_use(a->form);
+    const bool sums = !map && prism_sum_tc_use(a->form, a->precision);
     TcTable meta{};
     if (sums) rc = second_table(*c, a->form, a->degree, a->cell, PREC_TF32X3, &meta.image);
     else rc = tc_table(*c, a->form, a->degree, a->cell, a->precision, &meta);

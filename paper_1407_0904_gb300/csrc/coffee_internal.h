@@ -287,8 +287,8 @@ int launch_csr_map(const int32_t* l2g, int64_t ncells, int nloc, const int64_t* 
 int tc_csr_supported(int form, int degree, int cell, int precision);
 void build_prism_tc_image(int form, int degree, int prec, std::vector<uint8_t>& img, TcTable& meta);
 int launch_prism_tc(int form, int degree, const TcParams& p, int num_sms, void* stream, std::string& why);
-// the same forms with the quadrature summed in two steps (k_prism_sum_tc.cu): local assembly
-bool prism_sum_tc_use(int form);
+// the same with the quadrature summed in two steps (k_prism_sum_tc.cu): split-tf32 element matrices
+bool prism_sum_tc_use(int form, int precision);
 void build_prism_sum_image(int form, int degree, std::vector<uint8_t>& img);
 int launch_prism_sum_tc(int form, int degree, const TcParams& p, int num_sms, void* stream);
 int launch_tc_csr(int form, int cell, const TcParams& p, int num_sms, void* stream, std::string& why);

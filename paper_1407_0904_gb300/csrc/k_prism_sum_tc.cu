@@ -1,4 +1,4 @@
-// tcgen05 local assembly of HELMHOLTZ and ADVDIFF on prisms with the quadrature summed in two steps.
+// tcgen05 local assembly of HELMHOLTZ and ADVDIFF on prisms in split tf32 with the quadrature summed in two steps.
 //
 // Contracted over all points at once (k_prism_tc.cu) an element matrix takes K = 7 (k+2)^3 columns against
 // ((k+1)^2 (k+2) / 2)^2 outputs: 8.9 MFLOP of split-tf32 MMAs a P3 cell, whose 13 slices also need the factors
@@ -13,8 +13,8 @@
 // fields of w_q (g(x_q) - g_c) first, then one more "point" with the fields of g_c against the products summed
 // with the triangle's weights, so that the accumulator stays small while it is added to most often.
 //
-// Every precision runs the split-tf32 operands: the MMAs do not bound it (one pass instead of three saved 5-15 %),
-// and factors summed before they are rounded average their rounding errors less than single points do.
+// Only TF32X3: the other precisions are defined by the parts that each point's factors are held in, and sums over z
+// rounded to those parts are other numbers (TF32 here and there: 3e-4 of the entries apart).
 // Bound by shared memory (L1 data pipe 72 % busy beside the MMAs' operands, 78 of 7.5 KB a P3 tile) and, with it, the
 // latency of the fields' and the epilogue's chains: a seventh fewer wavefronts by padding gained 2 % at P3, lost 3 % at P1. Factors and fields are separate warps, two tiles of factors in flight,
 // because in the same warps one after the other they took 24,000 cycles a P3 tile for 16,800; matrix rows put
@@ -534,7 +534,7 @@ cudaError_t launch_zd(int degree, const TcParams& p, int num_sms, cudaStream_t s
 
 }  // namespace
 
-// All of both forms at any count. Graph-replayed times, us, split tf32, one contraction over all points | here:
+// TF32X3, both forms at any count. Graph-replayed times, us, one contraction over all points | here:
 //   cells                 7           3000          P1 250,000, P2 110,592, P3 55,296, P4 16,000
 //   HELMHOLTZ   P1    25 | 10       27 | 13       280 | 148
 //               P2    53 | 13       56 | 14       297 | 188
@@ -544,10 +544,11 @@ cudaError_t launch_zd(int degree, const TcParams& p, int num_sms, cudaStream_t s
 //               P2    75 | 14       77 | 20       417 | 316
 //               P3   643 | 17      626 | 32      1871 | 336
 //               P4  3306 | 25     3202 | 81      3210 | 381
-// The plain tf32 and bf16 operands of the other kernel: 267-391 us at P1, 258-387 at P2, 1104 and more above.
-// Its error against 64 bits is 1.7-4.8 times this one's in split tf32, 1.2-3.8 times in bf16x3.
-// MASS (K = (k+2)^3) and the CSR forms stay with the other.
-bool prism_sum_tc_use(int form) { return form == FORM_HELMHOLTZ || form == FORM_ADVDIFF; }
+// The error of one contraction against 64 bits is 1.7-4.8 times this one's.
+// MASS (K = (k+2)^3), the CSR forms and the other precisions stay with the other kernel.
+bool prism_sum_tc_use(int form, int precision) {
+  return (form == FORM_HELMHOLTZ || form == FORM_ADVDIFF) && precision == PREC_TF32X3;
+}
 
 // Chunks [chunk][part][NP rows x 64 B canonical] of the table T[o = it nt + jt][qt 8 + f] (after the last point the
 // products summed with the triangle's weights), then as floats the z products [QZ + 1][NR][4] (the last row summed

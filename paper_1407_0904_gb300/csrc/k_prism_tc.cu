@@ -1,5 +1,5 @@
-// tcgen05 assembly on prisms (the paper's third element shape, section 5.2): mass element matrices, and the global
-// CSR assembly of all three forms (the other two's element matrices: k_prism_sum_tc.cu).
+// tcgen05 assembly on prisms (the paper's third element shape, section 5.2): element matrices and the global CSR
+// assembly in every precision (split-tf32 element matrices of HELMHOLTZ and ADVDIFF: k_prism_sum_tc.cu).
 //
 // A prism's map is not affine, so the Jacobian is evaluated at every quadrature point and the
 // element matrix is a quadrature sum: A_e[o] = sum_{q,f} G_e[q][f] T[q*KQ+f][o] with
@@ -411,10 +411,9 @@ int pstages(const PGeom& g) {
 
 template <int PREC, int KQ>
 cudaError_t launch_p(const TcParams& p, int num_sms, cudaStream_t s, int nst, int smem) {
-  // element matrices of the other forms: k_prism_sum_tc.cu
   auto kern = k_assemble_prism_tc<PREC, KQ, true>;
-  if constexpr (KQ == 1) kern = p.map ? kern : k_assemble_prism_tc<PREC, KQ, false>;
-  else if (!p.map) return cudaErrorInvalidValue;
+  if constexpr (PREC != PREC_TF32X3 || KQ == 1) kern = p.map ? kern : k_assemble_prism_tc<PREC, KQ, false>;
+  else if (!p.map) return cudaErrorInvalidValue;  // k_prism_sum_tc.cu
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   if (e != cudaSuccess) return e;
   const int64_t ntiles = (p.ncells + BN - 1) / BN;
