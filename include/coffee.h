@@ -95,8 +95,11 @@ typedef enum {
  *   BF16:   T two bf16 parts, G one, two products;
  *   BF16X3: T and G three bf16 parts each, the six products of order <= 2.
  * FP64 runs on the CUDA cores, except where exact digit products on the tensor cores are faster
- * (triangles and tetrahedra: MASS on 10 or more nodes, HELMHOLTZ and ADVDIFF on 4 or more): every
- * operand as a fixed-point number of 61 or more bits, products and sums in integers, one rounding.
+ * (triangles and tetrahedra: MASS and HELMHOLTZ on 10 or more nodes, ADVDIFF on 4 or more): every
+ * operand as a fixed-point number of 61 or more bits below its cell's (entry's) largest, products
+ * and sums in integers, one rounding; entries without a term near the largest of their cell are
+ * summed in FP64 on the CUDA cores. Either way an entry's error is a few roundings of
+ * sum_k |G_e[k] T[k]|, the entry's own terms.
  * COFFEE_FLAG_CUDA_CORES keeps FP64 on the plain one-thread-per-cell kernel.
  * Parity bounds (max |A - A_exact| / max |A_exact| per cell): 1e-5 for TF32X3 and BF16X3,
  * 1e-2 for TF32 and BF16. */

@@ -137,6 +137,7 @@ struct DigitEntry {
   uint8_t* image = nullptr;
   int32_t* exps = nullptr;
   int32_t tk20[2] = {0, 0};
+  size_t emask = 0, groups = 0, classes = 0, weak = 0;  // offsets in exps (FP64 assembly)
 };
 
 struct DeviceCache {
@@ -216,10 +217,23 @@ int digit_table(DeviceCache& c, int form, int degree, int cell, Fp64Params& p) {
   auto it = c.digits.find(key);
   if (it == c.digits.end()) {
     std::vector<uint8_t> img;
-    std::vector<int32_t> y20;
+    Fp64Image h;
     DigitEntry ent;
-    build_fp64_image(form, degree, cell, img, y20, ent.tk20);
-    int rc = upload_digits(img, y20, ent);
+    build_fp64_image(form, degree, cell, img, h);
+    std::vector<int32_t> words = h.y20;
+    auto append = [&](const void* v, size_t bytes) {  // on 16 bytes
+      const size_t at = (words.size() + 3) & ~size_t(3);
+      words.resize(at + bytes / sizeof(int32_t));
+      std::memcpy(words.data() + at, v, bytes);
+      return at;
+    };
+    ent.emask = append(h.emask.data(), h.emask.size() * sizeof(uint32_t));
+    ent.groups = append(h.groups.data(), h.groups.size() * sizeof(int32_t));
+    ent.classes = append(h.classes.data(), h.classes.size() * sizeof(int32_t));
+    ent.weak = append(h.weak.data(), h.weak.size() * sizeof(double));
+    ent.tk20[0] = h.tk20[0];
+    ent.tk20[1] = h.tk20[1];
+    int rc = upload_digits(img, words, ent);
     if (rc != COFFEE_OK) return rc;
     it = c.digits.emplace(key, ent).first;
   }
@@ -227,6 +241,10 @@ int digit_table(DeviceCache& c, int form, int degree, int cell, Fp64Params& p) {
   p.yexp20 = it->second.exps;
   p.tk20[0] = it->second.tk20[0];
   p.tk20[1] = it->second.tk20[1];
+  p.emask = reinterpret_cast<const uint32_t*>(it->second.exps + it->second.emask);
+  p.groups = it->second.exps + it->second.groups;
+  p.classes = it->second.exps + it->second.classes;
+  p.weak = it->second.exps + it->second.weak;
   return COFFEE_OK;
 }
 

@@ -82,13 +82,23 @@ struct Fp64Params {
   const uint8_t* digits;  // tensor-core kernel: digit image of T, the entries' exponents and the scales
   const int32_t* yexp20;  // of the two kinds of factors (exponents << 20)
   int32_t tk20[2];
+  const uint32_t* emask;  // the entries' masks of large table entries, and the entries by mask (Fp64Image)
+  const int32_t *groups, *classes;
+  const void* weak;
 };
 // returns cudaError_t as int
 int launch_fp64(int form, int cell, const Fp64Params& p, void* stream);
 // FP64 on the tensor cores by exact digit products (k_fp64_tc.cu)
 int fp64_tc_use(int form, int degree, int cell);
-void build_fp64_image(int form, int degree, int cell, std::vector<uint8_t>& img, std::vector<int32_t>& y20,
-                      int32_t (&tk20)[2]);
+struct Fp64Image {  // beside the digit image of T
+  std::vector<int32_t> y20;      // exponent of every entry's row of T, << 20
+  int32_t tk20[2] = {0, 0};      // of the two kinds of terms
+  std::vector<uint32_t> emask;   // per entry, the k (of the first 32) whose |T[k]| is at least 1/8 of the largest
+  std::vector<int32_t> groups;   // per group of CTAs (k_fp64_tc.cu), its first and last + 1 in classes
+  std::vector<int32_t> classes;  // per distinct mask: mask, its entries' first and last + 1 row in weak, 0
+  std::vector<double> weak;      // a row per entry: T[k], zeros, the entry's number as the last word's bits
+};
+void build_fp64_image(int form, int degree, int cell, std::vector<uint8_t>& img, Fp64Image& h);
 int launch_fp64_tc(int form, int cell, const Fp64Params& p, int num_sms, void* stream);
 
 // ---- FP64 prism kernels (k_prism_sf.cu) ----

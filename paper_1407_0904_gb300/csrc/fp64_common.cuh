@@ -54,7 +54,6 @@ struct FormK {
                                                       : 1;
 };
 
-
 // The kind of term of factor k, 0 or 1 (factors of one kind have one order of magnitude): mass and
 // stiffness for HELMHOLTZ, stiffness and advection for ADVDIFF.
 template <int FORM, int D>
@@ -62,12 +61,25 @@ __host__ __device__ constexpr int term_of(int k) {
   return FORM == FORM_HELMHOLTZ ? (k > 0) : FORM == FORM_ADVDIFF ? (k >= (D + 1) * FormK<FORM, D>::P) : 0;
 }
 
-// The factors G[k] of cell e, false where an index is out of range (with p.validate). FAST: the
+// The factors of a cell: G[0..K) themselves, for ADVDIFF what they are products of: H (pairs a <= b), eps of the vertices, and
+// the advection terms (22 numbers for 36 factors on tetrahedra, which a thread can keep in registers).
+template <int FORM, int D>
+struct Factors {
+  static constexpr int NV = D + 1, P = D * (D + 1) / 2, K = FormK<FORM, D>::value;
+  static constexpr int COUNT = FORM == FORM_ADVDIFF ? P + NV + NV * D : K;
+  double f[COUNT];
+  __device__ __forceinline__ double at(int k) const {
+    if constexpr (FORM == FORM_ADVDIFF) return k < NV * P ? f[P + k / P] * f[k % P] : f[P + NV + k - NV * P];
+    else return f[k];
+  }
+};
+
+// The factors of cell e, false where an index is out of range (with p.validate). FAST: the
 // division by |det| as one reciprocal and a corrected product each (q + (s - q |det|) / |det|, which is
 // rounded as the division is but for rare last bits), instead of a division of about 20 instructions
 // per pair.
 template <int FORM, int D, bool FAST>
-__device__ __forceinline__ bool factors64(const Fp64Params& p, int64_t e, double (&G)[FormK<FORM, D>::value]) {
+__device__ __forceinline__ bool factors64(const Fp64Params& p, int64_t e, Factors<FORM, D>& G) {
   constexpr int NV = D + 1, P = D * (D + 1) / 2;
   int vid[NV], cid[NV];
   bool bad = false;
@@ -100,7 +112,7 @@ __device__ __forceinline__ bool factors64(const Fp64Params& p, int64_t e, double
   geometry64<D>(X, g);
   const double Dm = fabs(g.det);
   if constexpr (FORM == FORM_MASS) {
-    G[0] = Dm;
+    G.f[0] = Dm;
   } else {
     double H[P];  // |det| (K K^T)_{ab} = (adj adj^T)_{ab} / |det|, pairs a <= b
     const double inv = FAST ? 1.0 / Dm : 0.0;
@@ -120,21 +132,22 @@ __device__ __forceinline__ bool factors64(const Fp64Params& p, int64_t e, double
         }
       }
     if constexpr (FORM == FORM_HELMHOLTZ) {
-      G[0] = Dm;
+      G.f[0] = Dm;
 #pragma unroll
-      for (int k = 0; k < P; ++k) G[1 + k] = H[k];
+      for (int k = 0; k < P; ++k) G.f[1 + k] = H[k];
     } else {
       const double sg = g.det < 0.0 ? -1.0 : 1.0;
 #pragma unroll
-      for (int v = 0; v < NV; ++v) {
+      for (int k = 0; k < P; ++k) G.f[k] = H[k];
 #pragma unroll
-        for (int k = 0; k < P; ++k) G[v * P + k] = cf[v][0] * H[k];
+      for (int v = 0; v < NV; ++v) {
+        G.f[P + v] = cf[v][0];
 #pragma unroll
         for (int a = 0; a < D; ++a) {
           double s = 0.0;
 #pragma unroll
           for (int r = 0; r < D; ++r) s += (sg * g.adj[a][r]) * cf[v][1 + r];
-          G[NV * P + v * D + a] = s;
+          G.f[P + NV + v * D + a] = s;
         }
       }
     }
