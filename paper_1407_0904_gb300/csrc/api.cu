@@ -138,6 +138,7 @@ struct DigitEntry {
   int32_t* exps = nullptr;
   int32_t tk20[2] = {0, 0};
   size_t emask = 0, groups = 0, classes = 0, weak = 0;  // offsets in exps (FP64 assembly)
+  size_t large = 0, rows = 0;                            // the same (adjoint)
 };
 
 struct DeviceCache {
@@ -196,6 +197,14 @@ int fp64_table(DeviceCache& c, int form, int degree, int cell, const double** T)
   return COFFEE_OK;
 }
 
+// Words from v at the end of words, on 16 bytes: where they start
+size_t append_words(std::vector<int32_t>& words, const void* v, size_t bytes) {
+  const size_t at = (words.size() + 3) & ~size_t(3);
+  words.resize(at + bytes / sizeof(int32_t));
+  std::memcpy(words.data() + at, v, bytes);
+  return at;
+}
+
 // image followed by 32-bit exponents, uploaded as one allocation
 int upload_digits(std::vector<uint8_t>& img, const std::vector<int32_t>& exps, DigitEntry& ent) {
   const size_t at = (img.size() + 15) & ~size_t(15), bytes = at + exps.size() * sizeof(int32_t);
@@ -221,12 +230,7 @@ int digit_table(DeviceCache& c, int form, int degree, int cell, Fp64Params& p) {
     DigitEntry ent;
     build_fp64_image(form, degree, cell, img, h);
     std::vector<int32_t> words = h.y20;
-    auto append = [&](const void* v, size_t bytes) {  // on 16 bytes
-      const size_t at = (words.size() + 3) & ~size_t(3);
-      words.resize(at + bytes / sizeof(int32_t));
-      std::memcpy(words.data() + at, v, bytes);
-      return at;
-    };
+    auto append = [&](const void* v, size_t bytes) { return append_words(words, v, bytes); };
     ent.emask = append(h.emask.data(), h.emask.size() * sizeof(uint32_t));
     ent.groups = append(h.groups.data(), h.groups.size() * sizeof(int32_t));
     ent.classes = append(h.classes.data(), h.classes.size() * sizeof(int32_t));
@@ -253,15 +257,20 @@ int adjoint_table(DeviceCache& c, int form, int degree, int cell, BwdParams& p) 
   auto it = c.adjoint.find(key);
   if (it == c.adjoint.end()) {
     std::vector<uint8_t> img;
-    std::vector<int32_t> kexp20;
+    BwdImage h;
     DigitEntry ent;
-    build_backward_image(form, degree, cell, img, kexp20);
-    int rc = upload_digits(img, kexp20, ent);
+    build_backward_image(form, degree, cell, img, h);
+    std::vector<int32_t> words = h.kexp20;
+    ent.large = append_words(words, h.large.data(), h.large.size() * sizeof(uint32_t));
+    ent.rows = append_words(words, h.rows.data(), h.rows.size() * sizeof(double));
+    int rc = upload_digits(img, words, ent);
     if (rc != COFFEE_OK) return rc;
     it = c.adjoint.emplace(key, ent).first;
   }
   p.digits = it->second.image;
   p.kexp20 = it->second.exps;
+  p.large = reinterpret_cast<const uint32_t*>(it->second.exps + it->second.large);
+  p.rows = it->second.exps + it->second.rows;
   return COFFEE_OK;
 }
 

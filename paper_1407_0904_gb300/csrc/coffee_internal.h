@@ -142,10 +142,17 @@ struct BwdParams {
   int validate;
   const uint8_t* digits;  // tensor-core kernel: digit image of T and the factors' exponents (<< 20)
   const int32_t* kexp20;
+  const uint32_t* large;  // masks of T[k]'s large entries, and T by entry (BwdImage)
+  const void* rows;
 };
 // FP64 adjoint on the tensor cores by exact digit products (k_bwd_tc.cu)
 int backward_tc_use(int form, int degree, int cell);
-void build_backward_image(int form, int degree, int cell, std::vector<uint8_t>& img, std::vector<int32_t>& kexp20);
+struct BwdImage {  // beside the digit image of T
+  std::vector<int32_t> kexp20;  // exponent of every factor's row of T, << 20
+  std::vector<uint32_t> large;  // [rows read in pairs, singly][drain][k][4 words]: the o with |T[k][o]| >= 1/4 of the largest
+  std::vector<double> rows;     // T by entry, each entry's K numbers padded to an even count
+};
+void build_backward_image(int form, int degree, int cell, std::vector<uint8_t>& img, BwdImage& h);
 int launch_backward_tc(int form, int cell, const BwdParams& p, int num_sms, void* stream);
 int bwd_local_len(int form, int cell);
 int launch_backward(int form, int cell, const BwdParams& p, void* stream);

@@ -5,8 +5,8 @@
 // P2 on tetrahedra takes K N = 3600 of them per cell for Gbar and about 370 for the chain, 1.41 ms for 196,608
 // cells whose dA is read in 23 us. Here the contraction runs on the tensor cores over digits of dA (62-bit
 // fixed point, eight 8-bit digits), and the chain is rewritten on the adjugate A and the determinant
-// (K = A / det), about 280 operations: 0.204 ms. FP64 remains the bound there, now for the chain alone (0.11
-// ms) and for what does not overlap it; Helmholtz P2 (0.330 -> 0.130 ms) is bound by the making of the digits
+// (K = A / det), about 280 operations: 0.206 ms. FP64 remains the bound there, now for the chain alone (0.11
+// ms) and for what does not overlap it; Helmholtz P2 (0.326 -> 0.128 ms) is bound by the making of the digits
 // and the scan.
 //
 // Tiles of 128 cells on the TMEM lanes (M = 128), the factors k on the columns (16 or 48): per order d = p + q < 8
@@ -16,10 +16,15 @@
 // combined in 64-bit integers and rounded to double (with more than 112 entries the drains are added in FP64,
 // one rounding per 112 entries where the plain kernel rounds every one). Errors against 64-bit autograd are the
 // plain kernel's or smaller (1.0e-15 and 1.1e-15 for advection-diffusion P2).
+// An error relative to the largest dA of a row is a rounding of Gbar[k]'s own terms only if some large dA meets a large
+// T[k]. The scan looks for one for every k; cells without (one entry far above the others, a single row of dA) take
+// the plain sums, alone by the scan's warp (whole_cell), many by a lane each (plain_gbar, 1.1-1.2 times the plain
+// kernel's time when all are). The check costs up to a quarter: us for 196,608 tetrahedra without / with it, advection-
+// diffusion P1 164 / 221, P2 193 / 206, P3 584 / 670, Helmholtz P1 88 / 104, P2 124 / 128.
 //   warps 0-7    epilogue, two sets on alternate tiles (one drains while the other is in the FP64 chain);
 //                a thread has one cell: drains, chain rule, atomics or local rows
 //   warps 8-11   producers: digits of dA (this second reading of it hits L2)
-//   warps 12-14  scan: the largest exponent of each cell's dA
+//   warps 12-14  scan: the largest exponent of each cell's dA, the k with a large dA at a large T[k]
 //   warp 15      MMA issue
 #include <cuda_runtime.h>
 #include <algorithm>
@@ -48,6 +53,8 @@ constexpr int G_XRING = 4;           // drains whose cell exponents are kept
 constexpr int G_SH = 43;             // weight of order 0 in a drain's 64-bit sum (112 * 65^2 * 2^43 < 2^62)
 constexpr int G_ASTAGE = G_ND / 2 * G_CH * BM * 16;
 constexpr uint64_t G_BIAS = 0x8080808080808080ull;
+constexpr int CELL_PLAIN = INT32_MIN, CELL_DONE = INT32_MIN + 1;  // instead of an exponent: for plain_gbar; by the scan (whole_cell)
+constexpr int G_WEAK_A = 4, G_WEAK_T = 2;  // dA counts as large above 2^-4 of its drain's largest, T[k] above 2^-2 of its own
 
 struct alignas(8) GBars {
   uint64_t full[G_STAGES], empty[G_STAGES], tfull[2][2], tempty[2], xfull[G_XRING], xempty[G_XRING], done;  // tfull[set of warps][buffer]
@@ -64,6 +71,7 @@ struct Adj {
   static constexpr int STAGES = G_STAGES * STAGE <= 200 * 1024 ? G_STAGES : 3;
   static constexpr int NCF = FORM == FORM_ADVDIFF ? NV * (1 + D) : 0;
   static constexpr int NL = NV * D + NCF;
+  static constexpr int KP = (K + 1) / 2 * 2;                // words of an entry's row in the transposed T
 };
 
 // expects bytes in the barrier's current phase, without arriving (this thread's arrival follows its own stores)
@@ -118,15 +126,30 @@ __device__ __forceinline__ void store_pairs(uint8_t* dst, uint64_t U0, uint64_t 
   }
 }
 
-// Gbar of a cell whose dA the digits do not take (not finite, or outside 2^+-900)
+// Bit of entry o of a drain in the masks of large entries: 16 bits for each of the eight lanes that scan a row
+COFFEE_HD inline int mask_bit(int o, bool vec) { return vec ? o % 16 / 2 * 16 + o / 16 * 2 + o % 2 : o % 8 * 16 + o / 8; }
+
+// Gbar of a cell whose dA the digits do not take: not finite, outside 2^+-900, or without a large entry where some T[k] is
+// large. T's rows by entry: by factor, one such cell of P3 tetrahedra (N = 400) alone took 800,000 cycles, 36 lines an entry.
 template <int FORM, int D>
 __device__ __noinline__ void plain_gbar(const BwdParams& p, int64_t e, double* Gb) {
+  constexpr int K = Adj<FORM, D>::K, KP = Adj<FORM, D>::KP;
   const double* row = static_cast<const double*>(p.dout) + e * p.N;
-  for (int k = 0; k < Adj<FORM, D>::K; ++k) {
-    double s = 0.0;
-    for (int o = 0; o < p.N; ++o) s = fma(__ldg(p.T + (int64_t)k * p.N + o), __ldg(row + o), s);
-    Gb[k] = s;
+  const double2* T = static_cast<const double2*>(p.rows);
+  double s[KP];
+#pragma unroll
+  for (int k = 0; k < KP; ++k) s[k] = 0.0;
+  for (int o = 0; o < p.N; ++o) {
+    const double a = __ldg(row + o);
+#pragma unroll
+    for (int k = 0; k < KP; k += 2) {
+      const double2 t = __ldg(T + o * (KP / 2) + k / 2);
+      s[k] = fma(t.x, a, s[k]);
+      s[k + 1] = fma(t.y, a, s[k + 1]);
+    }
   }
+#pragma unroll
+  for (int k = 0; k < K; ++k) Gb[k] = s[k];
 }
 
 // Chain rule of one cell, from Gbar to the local gradient L (vertex coordinates v*D + r, then eps_v, then
@@ -244,6 +267,76 @@ __device__ __forceinline__ void chain_rule(const double (&X)[D + 1][D], const Bw
   }
 }
 
+// The local gradient from Gbar, to the cell's local row or added to the vertices' and coefficients' gradients
+template <int FORM, int D>
+__device__ __forceinline__ void finish_cell(const BwdParams& p, int64_t e, const int (&vid)[D + 1], const int (&cid)[D + 1],
+                                            const double (&X)[D + 1][D], const double (&Gb)[FormK<FORM, D>::value]) {
+  constexpr int NV = D + 1, NL = Adj<FORM, D>::NL;
+  double L[NL];
+  chain_rule<FORM, D>(X, p, cid, Gb, L);
+  if (p.local) {  // deterministic mode: summed later in cell order
+#pragma unroll
+    for (int j = 0; j < NL; ++j) p.local[e * NL + j] = L[j];
+  } else {
+#pragma unroll
+    for (int v = 0; v < NV; ++v)
+#pragma unroll
+      for (int r = 0; r < D; ++r) atomicAdd(p.d_coords + (int64_t)vid[v] * D + r, L[v * D + r]);
+    if constexpr (FORM == FORM_ADVDIFF) {
+      if (p.d_coef) {
+#pragma unroll
+        for (int v = 0; v < NV; ++v) {
+          double* dc = p.d_coef + (int64_t)cid[v] * (D + 1);
+          atomicAdd(dc, L[NV * D + v]);
+#pragma unroll
+          for (int r = 0; r < D; ++r) atomicAdd(dc + 1 + r, L[NV * D + NV + v * D + r]);
+        }
+      }
+    }
+  }
+}
+
+// One cell without digits by a whole warp. Alone in a warp of the epilogue it would hold up a tile (plain_gbar takes 700,000
+// cycles of latency for N = 400: with one cell in 10,000, advection-diffusion P3 on 196,608 tetrahedra took 1290 us,
+// now 670).
+template <int FORM, int D>
+__device__ __noinline__ void whole_cell(const BwdParams& p, int64_t e) {
+  constexpr int K = Adj<FORM, D>::K, NV = D + 1;
+  const double* row = static_cast<const double*>(p.dout) + e * p.N;
+  double Gb[K];
+#pragma unroll
+  for (int k = 0; k < K; ++k) Gb[k] = 0.0;
+  for (int o = threadIdx.x & 31; o < p.N; o += 32) {
+    const double a = __ldg(row + o);
+#pragma unroll
+    for (int k = 0; k < K; ++k) Gb[k] = fma(__ldg(p.T + (int64_t)k * p.N + o), a, Gb[k]);
+  }
+  __syncwarp();
+#pragma unroll
+  for (int k = 0; k < K; ++k)
+#pragma unroll
+    for (int m = 16; m > 0; m /= 2) Gb[k] += __shfl_xor_sync(0xffffffffu, Gb[k], m);
+  if ((threadIdx.x & 31) == 0) {
+    int vid[NV], cid[NV];
+    bool bad = false;  // (which the epilogue reports)
+#pragma unroll
+    for (int v = 0; v < NV; ++v) {
+      vid[v] = __ldg(p.c2v + e * NV + v);
+      cid[v] = FORM == FORM_ADVDIFF ? __ldg(p.c2d + e * NV + v) : 0;
+      if (p.validate && (vid[v] < 0 || vid[v] >= p.nverts || (FORM == FORM_ADVDIFF && (cid[v] < 0 || cid[v] >= p.ncoefnodes)))) bad = true;
+    }
+    if (!bad) {
+      double X[NV][D];
+#pragma unroll
+      for (int v = 0; v < NV; ++v)
+#pragma unroll
+        for (int r = 0; r < D; ++r) X[v][r] = __ldg(p.coords + (int64_t)vid[v] * D + r);
+      finish_cell<FORM, D>(p, e, vid, cid, X, Gb);
+    }
+  }
+  __syncwarp();
+}
+
 template <int FORM, int D>
 __global__ void __launch_bounds__(G_THREADS, 1) k_backward_tc(const BwdParams p) {
   using AF = Adj<FORM, D>;
@@ -251,13 +344,22 @@ __global__ void __launch_bounds__(G_THREADS, 1) k_backward_tc(const BwdParams p)
   extern __shared__ __align__(1024) uint8_t smem_raw[];
   uint8_t* sS = smem_raw;
   int* sX = reinterpret_cast<int*>(sS + AF::STAGES * AF::STAGE);
-  GBars* bars = reinterpret_cast<GBars*>(sX + G_XRING * BM);
+  uint4* sT = reinterpret_cast<uint4*>(sX + G_XRING * BM);            // masks of T's large entries [drain][k]
+  const int ndr = ((p.N + G_PE - 1) / G_PE + G_DRAIN - 1) / G_DRAIN;
+  uint4* sL = sT + ndr * K;                                           // of dA's, of the eight rows a scan warp is at
+  int4* sR = reinterpret_cast<int4*>(sL + G_SCAN * 8);                // a row's scale and factors so far [BM]
+  GBars* bars = reinterpret_cast<GBars*>(sR + BM);
 
   const int warp = __shfl_sync(0xffffffffu, (int)threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
   const int N = p.N;
-  const int nparts = (N + G_PE - 1) / G_PE, ndrains = (nparts + G_DRAIN - 1) / G_DRAIN;
+  const int nparts = (N + G_PE - 1) / G_PE, ndrains = ndr;
+  const bool vec = (N & 1) == 0 && (reinterpret_cast<uintptr_t>(p.dout) & 15) == 0;  // rows that can be read in pairs
   const int64_t ntiles = (p.ncells + BM - 1) / BM;
 
+  {
+    const uint4* src = reinterpret_cast<const uint4*>(p.large) + (vec ? 0 : ndrains * K);
+    for (int i = threadIdx.x; i < ndrains * K; i += G_THREADS) sT[i] = __ldg(src + i);
+  }
   if (threadIdx.x == 0) {
     for (int s = 0; s < G_STAGES; ++s) {
       mbar_init(smem_u32(&bars->full[s]), BM);
@@ -294,7 +396,6 @@ __global__ void __launch_bounds__(G_THREADS, 1) k_backward_tc(const BwdParams p)
     // (a lane per cell reads as many bytes, but every load then touches 32 lines: L1 took 1000 cycles a part)
     // (half warps store 128 contiguous bytes: rows 0-7, the chunk of pr 0 and 1 or of pr 2 and 3)
     const int w = warp - G_EPI, r8 = (lane >> 1) & 7, pr = (lane & 1) | (lane >> 4) << 1;
-    const bool vec = (N & 1) == 0 && (reinterpret_cast<uintptr_t>(p.dout) & 15) == 0;
     uint32_t n = 0, dr = 0;  // parts stored, drains begun
     bool ok = true;
     for (int64_t t = blockIdx.x; t < ntiles && ok; t += gridDim.x) {
@@ -348,15 +449,20 @@ __global__ void __launch_bounds__(G_THREADS, 1) k_backward_tc(const BwdParams p)
     }
   } else if (warp >= G_EPI + G_PROD && warp < G_WARPS - 1) {
     // ---------------- scan: the largest exponent of every cell's dA in a drain's entries, drains ahead ----------------
+    // A drain's error is 2^-55 of max|T[k]| times its own largest |dA|: no more than roundings of sum_o |T[k][o] dA[o]| where a
+    // drain of at least half that scale has a large dA at a large T[k]. So the scan also finds, per row and drain, the k for
+    // which one has (a lane per k, masks of 112 entries), and leaves cells with a k for which none has to plain_gbar.
     const int w = warp - (G_EPI + G_PROD);
-    const bool vec = (N & 1) == 0 && (reinterpret_cast<uintptr_t>(p.dout) & 15) == 0;
     const double* dA = static_cast<const double*>(p.dout);
     uint32_t dr = 0;
     bool ok = true;
     for (int64_t t = blockIdx.x; t < ntiles && ok; t += gridDim.x)
     for (int dn = 0; dn < ndrains; ++dn, ++dr) {
       const int r = (int)(dr % G_XRING), o1 = dn * (G_DRAIN * G_PE), len = min(N - o1, G_DRAIN * G_PE);
-      if (!mbar_wait(xempty + 8 * r, ((dr / G_XRING) & 1u) ^ 1u, p.err)) { ok = false; break; }
+      ok = __all_sync(0xffffffffu, mbar_wait(xempty + 8 * r, ((dr / G_XRING) & 1u) ^ 1u, p.err));
+      if (!ok) break;
+      const uint4 none = make_uint4(0, 0, 0, 0);
+      const uint4 t0 = lane < K ? sT[dn * K + lane] : none, t1 = lane + 32 < K ? sT[dn * K + lane + 32] : none;
       // Eight rows at a time, eight lanes each on two of them, and 16 predicated loads in flight: the scan is
       // bound by their latency (one row a time and a loop left to the compiler, which takes short rows one
       // load at a time, took 34,000 cycles a tile of 100 entries, half the kernel's time).
@@ -378,54 +484,99 @@ __global__ void __launch_bounds__(G_THREADS, 1) k_backward_tc(const BwdParams p)
             if (en + 4 < p.ncells) asm volatile("prefetch.global.L2 [%0];" ::"l"(nx + (int64_t)4 * N));
           }
         }
+        auto over_row = [&]() {
+#pragma unroll
+          for (int m = 1; m < 8; m *= 2)
+#pragma unroll
+            for (int j = 0; j < 2; ++j) {
+              X[j] = max(X[j], __shfl_xor_sync(0xffffffffu, X[j], m));
+              some[j] |= __shfl_xor_sync(0xffffffffu, some[j], m);
+            }
+        };
+        uint32_t large[2] = {0, 0};  // this lane's entries above 2^-4 of the row's largest
         if (vec) {
           const int o0 = 2 * (lane & 7);
-          {
-            int4 b[2][7];
+          int4 b[2][7];
 #pragma unroll
-            for (int j = 0; j < 7; ++j) {
-              b[0][j] = o0 + 16 * j < colsA ? __ldg(reinterpret_cast<const int4*>(src + o0 + 16 * j)) : make_int4(0, 0, 0, 0);
-              b[1][j] = o0 + 16 * j < colsB ? __ldg(reinterpret_cast<const int4*>(srcB + o0 + 16 * j)) : make_int4(0, 0, 0, 0);
-            }
+          for (int j = 0; j < 7; ++j) {
+            b[0][j] = o0 + 16 * j < colsA ? __ldg(reinterpret_cast<const int4*>(src + o0 + 16 * j)) : make_int4(0, 0, 0, 0);
+            b[1][j] = o0 + 16 * j < colsB ? __ldg(reinterpret_cast<const int4*>(srcB + o0 + 16 * j)) : make_int4(0, 0, 0, 0);
+          }
 #pragma unroll
-            for (int j = 0; j < 14; ++j) {
-              const int4 c = b[j & 1][j >> 1];
-              X[j & 1] = max(X[j & 1], max(c.y & 0x7FFFFFFF, c.w & 0x7FFFFFFF));
-              some[j & 1] |= c.x | c.z;
-            }
+          for (int j = 0; j < 14; ++j) {
+            const int4 c = b[j & 1][j >> 1];
+            X[j & 1] = max(X[j & 1], max(c.y & 0x7FFFFFFF, c.w & 0x7FFFFFFF));
+            some[j & 1] |= c.x | c.z;
+          }
+          over_row();
+#pragma unroll
+          for (int j = 0; j < 14; ++j) {
+            const int4 c = b[j & 1][j >> 1];
+            const int least = X[j & 1] - (G_WEAK_A << 20);
+            large[j & 1] |= ((c.y & 0x7FFFFFFF) >= least ? 1u << (j & ~1) : 0u) | ((c.w & 0x7FFFFFFF) >= least ? 2u << (j & ~1) : 0u);
           }
         } else {
           const int o0 = lane & 7;
-          {
-            int2 b[2][14];
+          int2 b[2][14];
 #pragma unroll
-            for (int j = 0; j < 14; ++j) {
-              b[0][j] = o0 + 8 * j < colsA ? __ldg(reinterpret_cast<const int2*>(src + o0 + 8 * j)) : make_int2(0, 0);
-              b[1][j] = o0 + 8 * j < colsB ? __ldg(reinterpret_cast<const int2*>(srcB + o0 + 8 * j)) : make_int2(0, 0);
-            }
+          for (int j = 0; j < 14; ++j) {
+            b[0][j] = o0 + 8 * j < colsA ? __ldg(reinterpret_cast<const int2*>(src + o0 + 8 * j)) : make_int2(0, 0);
+            b[1][j] = o0 + 8 * j < colsB ? __ldg(reinterpret_cast<const int2*>(srcB + o0 + 8 * j)) : make_int2(0, 0);
+          }
 #pragma unroll
-            for (int j = 0; j < 28; ++j) {
-              const int2 c = b[j & 1][j >> 1];
-              X[j & 1] = max(X[j & 1], c.y & 0x7FFFFFFF);
-              some[j & 1] |= c.x;
-            }
+          for (int j = 0; j < 28; ++j) {
+            const int2 c = b[j & 1][j >> 1];
+            X[j & 1] = max(X[j & 1], c.y & 0x7FFFFFFF);
+            some[j & 1] |= c.x;
+          }
+          over_row();
+#pragma unroll
+          for (int j = 0; j < 28; ++j)
+            large[j & 1] |= (b[j & 1][j >> 1].y & 0x7FFFFFFF) >= X[j & 1] - (G_WEAK_A << 20) ? 1u << (j >> 1) : 0u;
+        }
+        uint16_t* masks = reinterpret_cast<uint16_t*>(sL + w * 8);
+#pragma unroll
+        for (int j = 0; j < 2; ++j) masks[((lane >> 3) + 4 * j) * 8 + (lane & 7)] = (uint16_t)large[j];
+        __syncwarp();
+        uint32_t lo = 0, hi = 0;  // of row row0 + lane, lanes 0 to 7: the k with a large dA at a large T[k]
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+          const uint4 m = sL[w * 8 + j];
+          const uint32_t g0 = __ballot_sync(0xffffffffu, ((t0.x & m.x) | (t0.y & m.y) | (t0.z & m.z) | (t0.w & m.w)) != 0u);
+          if (lane == j) lo = g0;
+          if constexpr (K > 32) {
+            const uint32_t g1 = __ballot_sync(0xffffffffu, ((t1.x & m.x) | (t1.y & m.y) | (t1.z & m.z) | (t1.w & m.w)) != 0u);
+            if (lane == j) hi = g1;
           }
         }
-#pragma unroll
-        for (int m = 1; m < 8; m *= 2)
-#pragma unroll
-          for (int j = 0; j < 2; ++j) {
-            X[j] = max(X[j], __shfl_xor_sync(0xffffffffu, X[j], m));
-            some[j] |= __shfl_xor_sync(0xffffffffu, some[j], m);
+        const int xa = __shfl_sync(0xffffffffu, X[0], (lane & 3) * 8), xb = __shfl_sync(0xffffffffu, X[1], (lane & 3) * 8);
+        const int sa = __shfl_sync(0xffffffffu, some[0], (lane & 3) * 8), sb = __shfl_sync(0xffffffffu, some[1], (lane & 3) * 8);
+        bool fails = false;
+        if (lane < 8) {
+          const int x = lane & 4 ? xb : xa, any = lane & 4 ? sb : sa, ef = x & 0x7FF00000, row = row0 + lane;
+          const bool wild = (x | any) != 0 && (ef < (123 << 20) || ef > (1923 << 20));
+          // scale (exponent) and factors of the drains at it, or one below or above
+          int4 state = dn ? sR[row] : make_int4(0, -1, -1, 0);
+          if (ef != 0 && (state.x == 0 || ef >= state.x - (1 << 20))) {
+            const bool fresh = state.x == 0 || ef > state.x + (1 << 20);
+            state.y = (int)(lo | (fresh ? 0u : (uint32_t)state.y));
+            state.z = (int)(hi | (fresh ? 0u : (uint32_t)state.z));
+            state.x = fresh ? ef : state.x;
           }
-        if ((lane & 7) == 0) {
-#pragma unroll
-          for (int j = 0; j < 2; ++j) {
-            const int ef = X[j] & 0x7FF00000;
-            const bool wild = (X[j] | some[j]) != 0 && (ef < (123 << 20) || ef > (1923 << 20));
-            sX[r * BM + row + 4 * j] = wild ? INT32_MIN : ef - (1022 << 20);
-          }
+          if (dn + 1 < ndrains) sR[row] = state;
+          constexpr uint64_t all = (1ull << K) - 1;
+          const uint64_t good = ((uint64_t)(uint32_t)state.z << 32 | (uint32_t)state.y) & all;
+          fails = dn + 1 == ndrains && good != all;
+          sX[r * BM + row] = wild || fails ? CELL_PLAIN : ef - (1022 << 20);
+          fails = fails && !wild;
         }
+        const uint32_t f = __ballot_sync(0xffffffffu, fails);
+        if (f != 0u && (f & (f - 1)) == 0u) {  // one of eight rows: here and now; more of them are many, for the epilogue's lanes
+          const int row = row0 + __ffs(f) - 1;
+          whole_cell<FORM, D>(p, t * BM + row);
+          if (lane == 0) sX[r * BM + row] = CELL_DONE;
+        }
+        __syncwarp();
       }
       __syncwarp();
       if (lane == 0) mbar_arrive(xfull + 8 * r);
@@ -501,7 +652,7 @@ __global__ void __launch_bounds__(G_THREADS, 1) k_backward_tc(const BwdParams p)
 #pragma unroll
         for (int r = 0; r < D; ++r) X[v][r] = work ? __ldg(p.coords + (int64_t)vid[v] * D + r) : 0.0;
       double Gb[K];
-      bool wild = false;
+      bool wild = false, done = false;
       for (int dn = 0; dn < ndrains; ++dn) {
         const uint32_t dr = (uint32_t)(i * ndrains + dn), buf = dr % BUFS;
         if (!mbar_wait(tfull + 16 * set + 8 * buf, (phases >> buf) & 1u, p.err)) { ok = false; break; }
@@ -509,7 +660,8 @@ __global__ void __launch_bounds__(G_THREADS, 1) k_backward_tc(const BwdParams p)
         __syncwarp();
         tc_fence_after();
         const int x20 = sX[(dr % G_XRING) * BM + q * 32 + lane];
-        wild = wild || x20 == INT32_MIN;
+        wild = wild || x20 == CELL_PLAIN;
+        done = x20 == CELL_DONE;
         __syncwarp();
         if (lane == 0) mbar_arrive(xempty + 8 * (int)(dr % G_XRING));
 #pragma unroll
@@ -542,35 +694,14 @@ __global__ void __launch_bounds__(G_THREADS, 1) k_backward_tc(const BwdParams p)
         if (p.local)
           for (int j = 0; j < NL; ++j) p.local[e * NL + j] = 0.0;
       }
-      if (work) {
-        double L[NL];
+      if (work && !done) {
         if (wild) {
           double tmp[K];
           plain_gbar<FORM, D>(p, e, tmp);
 #pragma unroll
           for (int k = 0; k < K; ++k) Gb[k] = tmp[k];
         }
-        chain_rule<FORM, D>(X, p, cid, Gb, L);
-        if (p.local) {  // deterministic mode: summed later in cell order
-#pragma unroll
-          for (int j = 0; j < NL; ++j) p.local[e * NL + j] = L[j];
-        } else {
-#pragma unroll
-          for (int v = 0; v < NV; ++v)
-#pragma unroll
-            for (int r = 0; r < D; ++r) atomicAdd(p.d_coords + (int64_t)vid[v] * D + r, L[v * D + r]);
-          if constexpr (FORM == FORM_ADVDIFF) {
-            if (p.d_coef) {
-#pragma unroll
-              for (int v = 0; v < NV; ++v) {
-                double* dc = p.d_coef + (int64_t)cid[v] * (D + 1);
-                atomicAdd(dc, L[NV * D + v]);
-#pragma unroll
-                for (int r = 0; r < D; ++r) atomicAdd(dc + 1 + r, L[NV * D + NV + v * D + r]);
-              }
-            }
-          }
-        }
+        finish_cell<FORM, D>(p, e, vid, cid, X, Gb);
       }
       __syncwarp();
     }
@@ -587,7 +718,9 @@ __global__ void __launch_bounds__(G_THREADS, 1) k_backward_tc(const BwdParams p)
 
 template <int FORM, int D>
 cudaError_t launch_adj(const BwdParams& p, int num_sms, cudaStream_t s) {
-  int smem = Adj<FORM, D>::STAGES * Adj<FORM, D>::STAGE + G_XRING * BM * 4 + (int)sizeof(GBars) + 64;
+  constexpr int fixed = Adj<FORM, D>::STAGES * Adj<FORM, D>::STAGE + G_XRING * BM * 4 + G_SCAN * 8 * 16 + BM * 16 + (int)sizeof(GBars) + 64;
+  static_assert(fixed + 11 * Adj<FORM, D>::K * 16 <= 227 * 1024, "P4 tetrahedra have the most drains, 11");
+  const int ndrains = ((p.N + G_PE - 1) / G_PE + G_DRAIN - 1) / G_DRAIN, smem = fixed + ndrains * Adj<FORM, D>::K * 16;
   const int grid = (int)std::min<int64_t>((p.ncells + BM - 1) / BM, num_sms);
   auto kern = k_backward_tc<FORM, D>;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
@@ -597,16 +730,28 @@ cudaError_t launch_adj(const BwdParams& p, int num_sms, cudaStream_t s) {
 }
 
 template <int FORM, int D>
-void adj_image(int degree, int cell, std::vector<uint8_t>& img, std::vector<int32_t>& kexp20) {
+void adj_image(int degree, int cell, std::vector<uint8_t>& img, BwdImage& h) {
+  std::vector<int32_t>& kexp20 = h.kexp20;
   using AF = Adj<FORM, D>;
   const int ns = nnodes(cell, degree), N = ns * ns, nparts = (N + G_PE - 1) / G_PE;
   std::vector<double> T;
   reference_tensor(FORM, degree, cell, T);
   img.assign((size_t)nparts * AF::TSTAGE, 0);
   kexp20.assign(AF::K, 0);
+  const int len = G_DRAIN * G_PE, ndrains = (N + len - 1) / len;
+  h.large.assign((size_t)2 * ndrains * AF::K * 4, 0);
+  h.rows.assign((size_t)N * AF::KP, 0.0);
   for (int k = 0; k < AF::K; ++k) {
     double big = 0.0;
     for (int o = 0; o < N; ++o) big = std::max(big, std::fabs(T[(size_t)k * N + o]));
+    for (int o = 0; o < N; ++o) {
+      h.rows[(size_t)o * AF::KP + k] = T[(size_t)k * N + o];
+      if (std::fabs(T[(size_t)k * N + o]) < std::ldexp(big, -G_WEAK_T)) continue;
+      for (int v = 0; v < 2; ++v) {
+        const int bit = mask_bit(o % len, v == 0);
+        h.large[((size_t)(v * ndrains + o / len) * AF::K + k) * 4 + bit / 32] |= 1u << (bit % 32);
+      }
+    }
     int y = 0;
     if (big > 0) std::frexp(big, &y);
     kexp20[k] = (y - 12 - G_SH + 1054) * (1 << 20);  // order 0: leading digits of 2^-6 each, 2^43 in the sum
@@ -625,9 +770,9 @@ void adj_image(int degree, int cell, std::vector<uint8_t>& img, std::vector<int3
 
 }  // namespace
 
-// Where this kernel runs instead of the plain one: where it is the faster (us for 196,608 cells, this / plain).
-// Advection-diffusion everywhere: triangles P1 75 / 121 to P4 393 / 1243, tetrahedra P1 174 / 372 to P4 1870 /
-// 15,250; Helmholtz on tetrahedra, P1 94 / 120 to P4 1800 / 3100, and on triangles P2 76 / 92 and P3 120 / 192,
+// Where this kernel runs instead of the plain one: where it is the faster (us for 196,608 cells of random dA, this / plain).
+// Advection-diffusion everywhere: triangles P1 84 / 111 to P4 379 / 1230, tetrahedra P1 221 / 362, P2 206 / 1400, P3 670 /
+// 5100; Helmholtz on tetrahedra, P1 104 / 114 to P3 408 / 1066, and on triangles P2 76 / 85 and P3 118 / 185,
 // but not P1 (54 / 51) and P4 (380 / 371: 225 entries, rows that only 8-byte loads can take). The mass matrix
 // has one FMA an entry, which the FP64 pipe does as fast as its 2 x 8 bytes are read (tetrahedra P2 125 / 91).
 int backward_tc_use(int form, int degree, int cell) {
@@ -635,11 +780,11 @@ int backward_tc_use(int form, int degree, int cell) {
   return form == FORM_ADVDIFF;
 }
 
-void build_backward_image(int form, int degree, int cell, std::vector<uint8_t>& img, std::vector<int32_t>& kexp20) {
+void build_backward_image(int form, int degree, int cell, std::vector<uint8_t>& img, BwdImage& h) {
   const bool tri = cell == CELL_TRI;
   if (form == FORM_HELMHOLTZ)
-    tri ? adj_image<FORM_HELMHOLTZ, 2>(degree, cell, img, kexp20) : adj_image<FORM_HELMHOLTZ, 3>(degree, cell, img, kexp20);
-  else tri ? adj_image<FORM_ADVDIFF, 2>(degree, cell, img, kexp20) : adj_image<FORM_ADVDIFF, 3>(degree, cell, img, kexp20);
+    tri ? adj_image<FORM_HELMHOLTZ, 2>(degree, cell, img, h) : adj_image<FORM_HELMHOLTZ, 3>(degree, cell, img, h);
+  else tri ? adj_image<FORM_ADVDIFF, 2>(degree, cell, img, h) : adj_image<FORM_ADVDIFF, 3>(degree, cell, img, h);
 }
 
 int launch_backward_tc(int form, int cell, const BwdParams& p, int num_sms, void* stream) {
