@@ -16,13 +16,13 @@
 //
 // The FP64 pipe (2 FMAs per cycle and SM) bounds this as it did the sums over all points that stood here
 // before (Burgers Jacobian P2: 435,000 FMAs a cell, 33.7 ms for 27,648 cells; Helmholtz P2 145,000). The two
-// steps take 20 FMAs per quadruple and triangle point (Burgers; Helmholtz 8, advection-diffusion 11; with the
-// exchanged entries summed one by one 27, 13, 18), 40,000 in all for P2 where the direct sum takes 21 per entry and
+// steps take 22 FMAs per quadruple and triangle point (Burgers; Helmholtz 8, advection-diffusion 13; with the
+// exchanged entries summed one by one 27, 13, 18), 44,000 in all for P2 where the direct sum takes 21 per entry and
 // point. u and its derivatives at the points are formed the same way.
-// Measured, now / the exchanged entries one by one / the direct sums: Burgers Jacobian 27,648 P2 3.18 / 3.77 /
-// 33.65 ms (40,000 + 9,000 FMAs, 0.79 of the FP64 rate), 2000 P4 7.5 / 9.7 / 279 ms; 27,648 P2 Helmholtz 1.30 / 1.74 /
-// 7.62, advection-diffusion 1.80 / 2.40 / 9.81 ms. Now / the direct sums: residual P2 0.96 / 2.83, mass 0.32 / 1.24 ms;
-// 60,000 P1 Helmholtz 0.58 / 1.74 ms; 300 cells P1 16-36 us as launched from Python against 33-81, P4 0.05-1.1 ms
+// Measured, now / the exchanged entries one by one / the direct sums: Burgers Jacobian 27,648 P2 3.35 / 3.77 /
+// 33.65 ms (44,000 + 9,000 FMAs), P1 0.40 ms for 20,000, 300 P4 1.16 ms; 27,648 P2 Helmholtz 1.29 / 1.74 /
+// 7.62, advection-diffusion 1.97 / 2.40 / 9.81 ms. Now / the direct sums: residual P2 0.95 / 2.83, mass 0.31 / 1.24 ms;
+// 60,000 P1 Helmholtz 0.58 / 1.74 ms; 300 cells P1 16-36 us as launched from Python against 33-81, P4 0.05-1.2 ms
 // against 1.1-70.
 // A block holds one cell (P1: seven, residual P2: two), its factors and fields in shared memory, and several
 // blocks share an SM, so that one's table reads and barriers hide behind another's FMAs.
@@ -54,8 +54,8 @@ struct Sf {
   static constexpr int cell_doubles = Q * NF + S1 + XU + WZ;
   static constexpr int ZTAB = QZ * NZP * 4 + QZ * NZ * 2;  // z products and zeta, zeta' (shared by the block)
   static constexpr size_t smem = sizeof(double) * ((size_t)CELLS * cell_doubles + ZTAB) + 16 * sizeof(int);
-  // offsets in the host's table (prism_sf_table)
-  static constexpr int T_PSI = 0, T_TP = T_PSI + QT * NT * 3, T_ZP = T_TP + QT * 8 * NTP, T_PT = T_ZP + ZTAB;
+  // offsets in the host's table (prism_sum_table)
+  static constexpr int T_PSI = 0, T_TP = T_PSI + QT * NT * 3, T_ZP = T_TP + QT * 12 * NTP, T_PT = T_ZP + ZTAB;
 };
 
 // Geometry at a point: adjugate (K = adj / det) and determinant
@@ -99,7 +99,7 @@ __global__ void __launch_bounds__(Sf<FORM, DEG>::THREADS) k_prism_sf(const Prism
   int* sbad = reinterpret_cast<int*>(sZ + S::ZTAB);  // [CELLS]
   const int tid = threadIdx.x;
   const double* __restrict__ psi = p.T + S::T_PSI;  // [QT][NT][3]: psi, d_s, d_t
-  const double* __restrict__ tp = p.T + S::T_TP;    // [QT][8][NTP]
+  const double* __restrict__ tp = p.T + S::T_TP;    // [QT][12][NTP]
   const double* __restrict__ pt = p.T + S::T_PT;    // triangle points [QT][3] (s, t, weight), z [QZ][2] (z, weight)
   for (int i = tid; i < S::ZTAB; i += THREADS) sZ[i] = __ldg(p.T + S::T_ZP + i);
   const double* zl = sZ + QZ * NZP * 4;
@@ -271,10 +271,10 @@ __global__ void __launch_bounds__(Sf<FORM, DEG>::THREADS) k_prism_sf(const Prism
           for (int k = 0; k < NB; ++k) o[k] = m[k];
           o += NB;
           o[0] = ss, o[1] = st, o[2] = tt;
-          o[3] = (sz1 + sz2) + bs, o[4] = (tz1 + tz2) + bt;
-          o[5] = (sz1 - sz2) - bs, o[6] = (tz1 - tz2) - bt;
+          o[3] = sz1 + sz2, o[4] = tz1 + tz2;
+          o[5] = sz1 - sz2, o[6] = tz1 - tz2;
           if constexpr (S::BETA) {
-            o[7] = (sz1 - sz2) + bs, o[8] = (tz1 - tz2) + bt;
+            o[7] = bs, o[8] = bt;
             o[9] = zz + bz1, o[10] = zz + bz2;
           } else {
             o[7] = zz + m[0];
@@ -284,18 +284,23 @@ __global__ void __launch_bounds__(Sf<FORM, DEG>::THREADS) k_prism_sf(const Prism
       __syncthreads();
       // ---- sums over the triangle's points, one quadruple (it <= jt, iz <= jz) per thread. Exchanging it with jt
       // leaves P+, R+ = (d psi_it psi_jt + psi_it d psi_jt) / 2 as they are and turns the sign of P-, R-; exchanging
-      // iz with jz turns that of V_sz, V_tz (1) - (2). So with x the beta_s field the four entries are
-      //   C +- sum (sz1 - sz2 - x) P- + .. + sum (zz + bz1) T    and    C -+ sum (sz1 - sz2 + x) P- + .. + sum (zz + bz2) T,
-      // C the sum of the ss, st, tt terms and of (sz1 + sz2 + x) P+ + (tz1 + tz2 + y) R+, common to all. ----
+      // iz with jz turns that of V_sz, V_tz (1) - (2). So the four entries are
+      //   C +- G + v1 + y    and    C -+ G + v2 + y,   G = sum (sz1 - sz2) P- + (tz1 - tz2) R-,
+      // C the sum of the ss, st, tt terms and of (sz1 + sz2) P+ + (tz1 + tz2) R+, common to all. What a half sum adds
+      // and the difference takes away again, sz1 psi_it d psi_jt and so on, is of the size of the terms of V_sz that the
+      // entry has (the ratio is one of basis functions). The flow's terms y are no such pair: an entry has either
+      // beta_s d psi_it psi_jt or beta_s psi_it d psi_jt (y2, y1), and one of these may be zero (flow along an axis), so
+      // they are summed each (with half sums of them too, 3.18 ms for 3.35 of the Burgers Jacobian P2, entries of the diffusion alone were
+      // off by roundings of the flow's). ----
       for (int i = tid; i < nc * S::items; i += THREADS) {
         const int c = i / S::items, k = i % S::items, zp = k / NTP, tq = k % NTP;
-        double M[NB > 0 ? NB : 1], C = 0.0, G1 = 0.0, G2 = 0.0, v1 = 0.0, v2 = 0.0;
+        double M[NB > 0 ? NB : 1], C = 0.0, G = 0.0, v1 = 0.0, v2 = 0.0, y1 = 0.0, y2 = 0.0;
 #pragma unroll
         for (int x = 0; x < (NB > 0 ? NB : 1); ++x) M[x] = 0.0;
         const double* f = sS + c * S::S1 + zp * NFLD;
         const double* tt = tp + tq;
 #pragma unroll 2
-        for (int qt = 0; qt < QT; ++qt, f += NZP * NFLD, tt += 8 * NTP) {
+        for (int qt = 0; qt < QT; ++qt, f += NZP * NFLD, tt += 12 * NTP) {
           const double T = __ldg(tt);
 #pragma unroll
           for (int x = 0; x < NB; ++x) M[x] = fma(f[x], T, M[x]);
@@ -304,9 +309,10 @@ __global__ void __launch_bounds__(Sf<FORM, DEG>::THREADS) k_prism_sf(const Prism
             const double Pp = __ldg(tt + 4 * NTP), Pm = __ldg(tt + 5 * NTP), Rp = __ldg(tt + 6 * NTP), Rm = __ldg(tt + 7 * NTP);
             C = fma(h[0], __ldg(tt + NTP), fma(h[1], __ldg(tt + 2 * NTP), fma(h[2], __ldg(tt + 3 * NTP), C)));
             C = fma(h[3], Pp, fma(h[4], Rp, C));
-            G1 = fma(h[5], Pm, fma(h[6], Rm, G1));
+            G = fma(h[5], Pm, fma(h[6], Rm, G));
             if constexpr (S::BETA) {
-              G2 = fma(h[7], Pm, fma(h[8], Rm, G2));
+              y1 = fma(h[7], __ldg(tt + 9 * NTP), fma(h[8], __ldg(tt + 11 * NTP), y1));
+              y2 = fma(h[7], __ldg(tt + 8 * NTP), fma(h[8], __ldg(tt + 10 * NTP), y2));
               v1 = fma(h[9], T, v1);
               v2 = fma(h[10], T, v2);
             } else {
@@ -316,7 +322,6 @@ __global__ void __launch_bounds__(Sf<FORM, DEG>::THREADS) k_prism_sf(const Prism
             C = fma(f[0], T, C);
           }
         }
-        if constexpr (!S::BETA) G2 = G1;
         if (sbad[c]) continue;
         int jt = 0, jz = 0;  // tq = jt (jt + 1) / 2 + it, zp = jz (jz + 1) / 2 + iz
         while ((jt + 1) * (jt + 2) / 2 <= tq) ++jt;
@@ -340,10 +345,10 @@ __global__ void __launch_bounds__(Sf<FORM, DEG>::THREADS) k_prism_sf(const Prism
               }
             }
         };
-        put(iz * NT + it, jz * NT + jt, C + G1 + v1);
-        if (it != jt) put(iz * NT + jt, jz * NT + it, C - G1 + v1);
-        if (iz != jz) put(jz * NT + it, iz * NT + jt, C - G2 + v2);
-        if (it != jt && iz != jz) put(jz * NT + jt, iz * NT + it, C + G2 + v2);
+        put(iz * NT + it, jz * NT + jt, (C + G) + (v1 + y1));
+        if (it != jt) put(iz * NT + jt, jz * NT + it, (C - G) + (v1 + y2));
+        if (iz != jz) put(jz * NT + it, iz * NT + jt, (C - G) + (v2 + y1));
+        if (it != jt && iz != jz) put(jz * NT + jt, iz * NT + it, (C + G) + (v2 + y2));
       }
     } else {
       // ---- residual: sums over z of a_c zeta + gamma_cz zeta', gamma_cs zeta, gamma_ct zeta, then over qt ----

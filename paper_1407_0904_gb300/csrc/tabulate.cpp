@@ -388,8 +388,8 @@ void prism_factor_tables(int form, int k, std::vector<double>& pts, std::vector<
 // Tables of the direction-by-direction sums over a prism's points (p per direction; qt over the triangle's
 // p^2, qz over z's p), nt triangle and k+1 interval functions, pairs (i <= j) numbered j (j+1)/2 + i:
 //   [qt][nt][3]      psi, d_s psi, d_t psi
-//   [qt][8][pairs]   psi_i psi_j; the d_s d_s, (d_s d_t + d_t d_s), d_t d_t products; half the sum and the difference
-//                    of d_s psi_i psi_j and psi_i d_s psi_j; the same with d_t
+//   [qt][12][pairs]  psi_i psi_j; the d_s d_s, (d_s d_t + d_t d_s), d_t d_t products; half the sum and the difference
+//                    of d_s psi_i psi_j and psi_i d_s psi_j; the same with d_t; these four products themselves
 //   [qz][pairs][4]   zeta_i zeta_j, zeta_i zeta'_j, zeta_j zeta'_i, zeta'_i zeta'_j
 //   [qz][k+1][2]     zeta, zeta'
 //   [qt][3], [qz][2] points and weights (s, t, weight), (z, weight)
@@ -401,14 +401,15 @@ void prism_sum_table(int form, int k, std::vector<double>& tab) {
   for (size_t i = 0; i < psi.size(); ++i)
     for (double v : {psi[i], dpsi[i * 2], dpsi[i * 2 + 1]}) tab.push_back(v);
   for (int qt = 0; qt < p * p; ++qt)
-    for (int kind = 0; kind < 8; ++kind)
+    for (int kind = 0; kind < 12; ++kind)
       for (int j = 0; j < nt; ++j)
         for (int i = 0; i <= j; ++i) {
           const double a = psi[(size_t)qt * nt + i], b = psi[(size_t)qt * nt + j];
           const double *da = &dpsi[((size_t)qt * nt + i) * 2], *db = &dpsi[((size_t)qt * nt + j) * 2];
-          const double v[8] = {a * b,     da[0] * db[0], da[0] * db[1] + da[1] * db[0], da[1] * db[1],
-                               (da[0] * b + a * db[0]) / 2, (da[0] * b - a * db[0]) / 2,
-                               (da[1] * b + a * db[1]) / 2, (da[1] * b - a * db[1]) / 2};
+          const double v[12] = {a * b,     da[0] * db[0], da[0] * db[1] + da[1] * db[0], da[1] * db[1],
+                                (da[0] * b + a * db[0]) / 2, (da[0] * b - a * db[0]) / 2,
+                                (da[1] * b + a * db[1]) / 2, (da[1] * b - a * db[1]) / 2,
+                                da[0] * b, a * db[0], da[1] * b, a * db[1]};
           tab.push_back(v[kind]);
         }
   for (int q = 0; q < p; ++q)
