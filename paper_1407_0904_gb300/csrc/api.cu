@@ -170,6 +170,25 @@ int device_cache(DeviceCache** out) {
   return COFFEE_OK;
 }
 
+// A table for the process's lifetime
+int upload(const void* h, size_t bytes, const char* what, void** out) {
+  void* d = nullptr;
+  cudaError_t e = cudaMalloc(&d, bytes);
+  if (e != cudaSuccess) return cuda_fail(e, (std::string("cudaMalloc(") + what + ")").c_str());
+  e = cudaMemcpy(d, h, bytes, cudaMemcpyHostToDevice);
+  if (e != cudaSuccess) {
+    cudaFree(d);
+    return cuda_fail(e, (std::string("cudaMemcpy(") + what + ")").c_str());
+  }
+  *out = d;
+  return COFFEE_OK;
+}
+
+int digit_table(DeviceCache& c, int form, int degree, int cell, Fp64Params& p);
+int adjoint_table(DeviceCache& c, int form, int degree, int cell, BwdParams& p);
+
+// T in FP64, and with it the digit images of the kernels that a later call of any size may take, in either
+// direction: after one call none allocates, so that it can be captured
 int fp64_table(DeviceCache& c, int form, int degree, int cell, const double** T) {
   form = table_form(form);
   auto key = std::make_tuple(form, degree, cell);
@@ -184,17 +203,16 @@ int fp64_table(DeviceCache& c, int form, int degree, int cell, const double** T)
   } else {
     reference_tensor(form, degree, cell, h);
   }
-  double* d = nullptr;
-  cudaError_t e = cudaMalloc(&d, h.size() * sizeof(double));
-  if (e != cudaSuccess) return cuda_fail(e, "cudaMalloc(reference tensor)");
-  e = cudaMemcpy(d, h.data(), h.size() * sizeof(double), cudaMemcpyHostToDevice);
-  if (e != cudaSuccess) {
-    cudaFree(d);
-    return cuda_fail(e, "cudaMemcpy(reference tensor)");
-  }
-  c.fp64[key] = d;
-  *T = d;
-  return COFFEE_OK;
+  void* d = nullptr;
+  int rc = upload(h.data(), h.size() * sizeof(double), "reference tensor", &d);
+  if (rc != COFFEE_OK) return rc;
+  c.fp64[key] = static_cast<double*>(d);
+  *T = static_cast<double*>(d);
+  if (cell == CELL_PRISM) return COFFEE_OK;
+  Fp64Params fp{};
+  BwdParams bp{};
+  if (fp64_tc_use(form, degree, cell) && (rc = digit_table(c, form, degree, cell, fp)) != COFFEE_OK) return rc;
+  return backward_tc_use(form, degree, cell) ? adjoint_table(c, form, degree, cell, bp) : COFFEE_OK;
 }
 
 // Words from v at the end of words, on 16 bytes: where they start
@@ -210,13 +228,10 @@ int upload_digits(std::vector<uint8_t>& img, const std::vector<int32_t>& exps, D
   const size_t at = (img.size() + 15) & ~size_t(15), bytes = at + exps.size() * sizeof(int32_t);
   img.resize(bytes);
   std::memcpy(img.data() + at, exps.data(), exps.size() * sizeof(int32_t));
-  cudaError_t e = cudaMalloc(&ent.image, bytes);
-  if (e != cudaSuccess) return cuda_fail(e, "cudaMalloc(digit table)");
-  e = cudaMemcpy(ent.image, img.data(), bytes, cudaMemcpyHostToDevice);
-  if (e != cudaSuccess) {
-    cudaFree(ent.image);
-    return cuda_fail(e, "cudaMemcpy(digit table)");
-  }
+  void* d = nullptr;
+  const int rc = upload(img.data(), bytes, "digit table", &d);
+  if (rc != COFFEE_OK) return rc;
+  ent.image = static_cast<uint8_t*>(d);
   ent.exps = reinterpret_cast<int32_t*>(ent.image + at);
   return COFFEE_OK;
 }
@@ -274,27 +289,6 @@ int adjoint_table(DeviceCache& c, int form, int degree, int cell, BwdParams& p) 
   return COFFEE_OK;
 }
 
-int tc_table(DeviceCache& c, int form, int degree, int cell, int prec, TcTable* meta) {
-  auto key = std::make_tuple(form, degree, cell, prec);
-  auto it = c.tc.find(key);
-  if (it == c.tc.end()) {
-    std::vector<uint8_t> img;
-    TcEntry ent;
-    build_tc_image(form, degree, cell, prec, img, ent.meta);
-    cudaError_t e = cudaMalloc(&ent.image, img.size());
-    if (e != cudaSuccess) return cuda_fail(e, "cudaMalloc(tensor-core table)");
-    e = cudaMemcpy(ent.image, img.data(), img.size(), cudaMemcpyHostToDevice);
-    if (e != cudaSuccess) {
-      cudaFree(ent.image);
-      return cuda_fail(e, "cudaMemcpy(tensor-core table)");
-    }
-    ent.meta.image = ent.image;
-    it = c.tc.emplace(key, ent).first;
-  }
-  *meta = it->second.meta;
-  return COFFEE_OK;
-}
-
 // A second operand image of T for one (form, degree, cell, precision): the sector-aligned stores' on simplices, the
 // two-step sums' on prisms.
 int second_table(DeviceCache& c, int form, int degree, int cell, int prec, const uint8_t** image) {
@@ -304,17 +298,35 @@ int second_table(DeviceCache& c, int form, int degree, int cell, int prec, const
     std::vector<uint8_t> img;
     if (cell == CELL_PRISM) build_prism_sum_image(form, degree, img);
     else build_shift_image(form, degree, cell, prec, img);
-    uint8_t* d = nullptr;
-    cudaError_t e = cudaMalloc(&d, img.size());
-    if (e != cudaSuccess) return cuda_fail(e, "cudaMalloc(second table)");
-    e = cudaMemcpy(d, img.data(), img.size(), cudaMemcpyHostToDevice);
-    if (e != cudaSuccess) {
-      cudaFree(d);
-      return cuda_fail(e, "cudaMemcpy(second table)");
-    }
-    it = c.second.emplace(key, d).first;
+    void* d = nullptr;
+    const int rc = upload(img.data(), img.size(), "second table", &d);
+    if (rc != COFFEE_OK) return rc;
+    it = c.second.emplace(key, static_cast<uint8_t*>(d)).first;
   }
   *image = it->second;
+  return COFFEE_OK;
+}
+
+// The operand image, and with it the second one where a call of another size, stride or kind (local, global) may take
+// it (see fp64_table)
+int tc_table(DeviceCache& c, int form, int degree, int cell, int prec, TcTable* meta) {
+  auto key = std::make_tuple(form, degree, cell, prec);
+  auto it = c.tc.find(key);
+  if (it == c.tc.end()) {
+    std::vector<uint8_t> img;
+    TcEntry ent;
+    build_tc_image(form, degree, cell, prec, img, ent.meta);
+    void* d = nullptr;
+    int rc = upload(img.data(), img.size(), "tensor-core table", &d);
+    if (rc != COFFEE_OK) return rc;
+    ent.image = static_cast<uint8_t*>(d);
+    ent.meta.image = ent.image;
+    it = c.tc.emplace(key, ent).first;
+    const uint8_t* second = nullptr;
+    if (cell == CELL_PRISM ? prism_sum_tc_use(form, prec) : tc_shift_possible(form, degree, cell, prec) != 0)
+      if ((rc = second_table(c, form, degree, cell, prec, &second)) != COFFEE_OK) return rc;
+  }
+  *meta = it->second.meta;
   return COFFEE_OK;
 }
 
@@ -370,9 +382,8 @@ int assemble_impl(const coffee_assemble_args* a, const uint32_t* map, int64_t nn
       return fail(COFFEE_ERR_UNSUPPORTED, "tensor-core prisms: MASS, HELMHOLTZ and ADVDIFF, P1-P4");
     const bool sums = !map && prism_sum_tc_use(a->form, a->precision);
     TcTable meta{};
-    if (sums) rc = second_table(*c, a->form, a->degree, a->cell, PREC_TF32X3, &meta.image);
-    else rc = tc_table(*c, a->form, a->degree, a->cell, a->precision, &meta);
-    if (rc != COFFEE_OK) return rc;
+    if ((rc = tc_table(*c, a->form, a->degree, a->cell, a->precision, &meta)) != COFFEE_OK) return rc;
+    if (sums && (rc = second_table(*c, a->form, a->degree, a->cell, a->precision, &meta.image)) != COFFEE_OK) return rc;
     TcParams p{};
     p.coords = a->coords;
     p.c2v = a->cell2vert;

@@ -222,6 +222,7 @@ int launch_tc_staged(int form, int cell, const TcParams& q, int num_sms, void* s
 int launch_tc(int form, int cell, const TcParams& p, int num_sms, void* stream, std::string& why);
 // sector-aligned stores (k_tc_shift.cu): whether element matrices of this form, stride and precision take them, and the
 // image of T^T that they need (per part, 16-byte K chunk and row: 8 zero rows, then the outputs)
+int tc_shift_possible(int form, int degree, int cell, int precision);
 int tc_shift_use(int form, int degree, int cell, int precision, int64_t ostride, unsigned tune, int64_t ncells);
 void build_shift_image(int form, int degree, int cell, int precision, std::vector<uint8_t>& img);
 int launch_tc_shift(int form, int cell, const TcParams& p, int num_sms, void* stream);

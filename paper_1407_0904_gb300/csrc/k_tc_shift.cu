@@ -239,18 +239,31 @@ cudaError_t launch_shift_prec(const TcParams& p, int num_sms, cudaStream_t s, in
 //   tris mm = 3       10 / 7.6   11 / 11    17 / 17    40 / 43    86 / 125
 //   tris mm = 6       12 / 7.8   13 / 11    21 / 18    50 / 40    109 / 93
 // Few cells do not fill tiles of 256 in eight classes, and with few slices the MMAs take longer than the stores.
-int tc_shift_use(int form, int degree, int cell, int precision, int64_t ostride, unsigned tune, int64_t ncells) {
-  if (!(form == FORM_MASS || form == FORM_HELMHOLTZ || form == FORM_ADVDIFF) || cell == CELL_PRISM || ostride % 8 == 0 ||
-      (tune & TUNE_STAGED_STORE))
-    return 0;
+namespace {
+struct ShiftShape {
+  int mtiles, mm;  // slices of 128 entries, MMAs an accumulator
+  bool fits;
+};
+ShiftShape shift_shape(int form, int degree, int cell, int precision) {
   const bool tf32 = precision == PREC_TF32 || precision == PREC_TF32X3;
-  const int kstep = tf32 ? 8 : 16, K = form_K(form, degree, cell), ksteps = (K + kstep - 1) / kstep, kbytes = ksteps * 32;
+  const int kstep = tf32 ? 8 : 16, K = form_K(form, degree, cell), ksteps = (K + kstep - 1) / kstep;
   const int ns = nnodes(cell, degree), N = ns * ns, mtiles = (N + BM - 1) / BM;
   const int passes = precision == PREC_TF32 ? 1 : precision == PREC_BF16 ? 2 : precision == PREC_TF32X3 ? 3 : 6;
-  const int mm = ksteps * passes;
-  if (mm > 3 && mtiles <= 4) return 0;
-  const int64_t least = mtiles > 4 ? (mm > 3 ? 32768 : 16384) : mm == 3 ? 131072 : 16384;
-  return ncells >= least && mtiles > 1 && N + 7 <= mtiles * BM && shift_smem(mtiles, kbytes, precision) <= 227 * 1024;
+  return {mtiles, ksteps * passes, mtiles > 1 && N + 7 <= mtiles * BM && shift_smem(mtiles, ksteps * 32, precision) <= 227 * 1024};
+}
+}  // namespace
+
+// whether some count of cells and stride takes this kernel
+int tc_shift_possible(int form, int degree, int cell, int precision) {
+  if (!(form == FORM_MASS || form == FORM_HELMHOLTZ || form == FORM_ADVDIFF) || cell == CELL_PRISM || precision == PREC_FP64) return 0;
+  const ShiftShape s = shift_shape(form, degree, cell, precision);
+  return s.fits && !(s.mm > 3 && s.mtiles <= 4);
+}
+
+int tc_shift_use(int form, int degree, int cell, int precision, int64_t ostride, unsigned tune, int64_t ncells) {
+  if (!tc_shift_possible(form, degree, cell, precision) || ostride % 8 == 0 || (tune & TUNE_STAGED_STORE)) return 0;
+  const ShiftShape s = shift_shape(form, degree, cell, precision);
+  return ncells >= (s.mtiles > 4 ? (s.mm > 3 ? 32768 : 16384) : s.mm == 3 ? 131072 : 16384);
 }
 
 void build_shift_image(int form, int degree, int cell, int prec, std::vector<uint8_t>& img) {
