@@ -170,12 +170,14 @@ int device_cache(DeviceCache** out) {
   return COFFEE_OK;
 }
 
-// A table for the process's lifetime
+// A table for the process's lifetime. The kernels that read it run on streams of the caller's, which may not wait for
+// the default stream, and a copy from pageable memory may return before it has arrived: wait for it here, once.
 int upload(const void* h, size_t bytes, const char* what, void** out) {
   void* d = nullptr;
   cudaError_t e = cudaMalloc(&d, bytes);
   if (e != cudaSuccess) return cuda_fail(e, (std::string("cudaMalloc(") + what + ")").c_str());
   e = cudaMemcpy(d, h, bytes, cudaMemcpyHostToDevice);
+  if (e == cudaSuccess) e = cudaStreamSynchronize(cudaStreamLegacy);
   if (e != cudaSuccess) {
     cudaFree(d);
     return cuda_fail(e, (std::string("cudaMemcpy(") + what + ")").c_str());
