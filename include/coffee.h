@@ -161,6 +161,11 @@ typedef enum {
  * bound. */
 #define COFFEE_FLAG_BURGERS_BLOCKS 2048u
 #define COFFEE_FLAG_BURGERS_FACTORED 4096u
+/* Large launches of element matrices that start off the 32-byte sectors (P4, padded rows of other strides) have a
+ * kernel of their own without these knobs, whose stores cover whole sectors. OUTPUT_LANES, TWO_STAGES, SUBTILE_*,
+ * CELL_LANES and STAGED_STORE ask for the other one, unless KNOB_HINT says that they are only how it is to run
+ * where the library takes it (the autotuner's choice). */
+#define COFFEE_FLAG_KNOB_HINT 8192u
 
 /* Number of rows of the element matrix (or length of the element vector): (k+1)(k+2)/2
  * (triangle), (k+1)(k+2)(k+3)/6 (tetrahedron) or (k+1)^2(k+2)/2 (prism), times d for

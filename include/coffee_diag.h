@@ -36,6 +36,11 @@ int coffee_diag_wait_timeout(coffee_stream_t stream);
 int coffee_table_image(int form, int degree, int cell, int precision, uint8_t* img, int64_t* nbytes,
                        int64_t* meta);
 
+/* Whether local assembly of ncells cells takes the kernel whose stores cover whole 32-byte sectors (1) or not (0):
+ * host-only, for tests of its rule. out_stride as in coffee_assemble_args (0: contiguous). */
+int coffee_diag_sector_stores(int form, int degree, int cell, int precision, unsigned flags, int64_t out_stride,
+                              int64_t ncells);
+
 #ifdef __cplusplus
 }
 #endif

@@ -28,6 +28,7 @@ FLAG_TENSOR_CORES = 512  # small element matrices: force the tcgen05 kernel
 FLAG_CUDA_CORES = 1024   # small element matrices: force the FP32 CUDA-core kernel
 FLAG_BURGERS_BLOCKS = 2048    # Burgers Jacobian: the block form (every block over [T1|T2|T3])
 FLAG_BURGERS_FACTORED = 4096  # Burgers Jacobian: the factored form (T1 against u, P in the epilogue)
+FLAG_KNOB_HINT = 8192    # the knobs are the autotuner's: they do not keep a launch from the sector-aligned stores
 
 FORM_NAMES = {MASS: "mass", HELMHOLTZ: "helmholtz", ADVDIFF: "advdiff", BURGERS_JAC: "burgers_jac",
               BURGERS_RESIDUAL: "burgers_residual"}
@@ -163,6 +164,15 @@ def diag_wait_timeout(stream=None):
     L = lib()
     L.coffee_diag_wait_timeout.argtypes = [ctypes.c_void_p]
     _check(L.coffee_diag_wait_timeout(_stream_handle(stream)))
+
+
+def diag_sector_stores(form, degree, cell, precision, flags=0, out_stride=0, ncells=0):
+    """Whether local assembly of ncells cells takes the kernel with sector-aligned stores (coffee_diag_sector_stores)."""
+    L = lib()
+    L.coffee_diag_sector_stores.argtypes = [ctypes.c_int] * 4 + [ctypes.c_uint, ctypes.c_int64, ctypes.c_int64]
+    r = L.coffee_diag_sector_stores(form, degree, cell, precision, flags, out_stride, ncells)
+    _check(min(r, 0))
+    return r == 1
 
 
 def peak_fp64():
@@ -341,8 +351,9 @@ def assemble(form, degree, cell, coords, cell2vert, coef=None, cell2dof=None, pr
              out_stride=None):
     """Element matrices [ncells, ndof, ndof] (float64 for FP64, float32 otherwise) on the device.
 
-    tune: FLAG_OUTPUT_LANES / FLAG_TWO_STAGES knobs; None uses the autotuner's choice for
-    this (form, degree, cell, precision) when one is cached, else the library default.
+    tune: FLAG_OUTPUT_LANES / FLAG_TWO_STAGES and the other knobs; None uses the autotuner's choice for
+    this (form, degree, cell, precision) when one is cached, else the library default, as hints
+    (FLAG_KNOB_HINT).
     coords_split: the (hi, lo) float pairs of coords (split_coords), optional.
     coef_f32: coef rounded to floats (round_coef), optional.
     out_stride: entries between consecutive element matrices (padded rows, e.g. a multiple of 32
@@ -378,8 +389,8 @@ def _tuned_flags(form, degree, cell, precision):
             _tune_cache = {}
     ent = _tune_cache.get("%d/%d/%d/%d" % (form, degree, cell, precision))
     if ent is not None:
-        return int(ent.get("flags", 0))
-    return _model_flags(form, degree, cell, precision)
+        return int(ent.get("flags", 0)) | FLAG_KNOB_HINT
+    return _model_flags(form, degree, cell, precision) | FLAG_KNOB_HINT
 
 
 @functools.lru_cache(maxsize=256, typed=True)

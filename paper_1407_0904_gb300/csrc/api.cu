@@ -369,6 +369,19 @@ int check_args(const coffee_assemble_args* a) {
   return COFFEE_OK;
 }
 
+unsigned tune_bits(unsigned flags) {
+  return ((flags & COFFEE_FLAG_OUTPUT_LANES) ? TUNE_OUTPUT_LANES : 0u) |
+         ((flags & COFFEE_FLAG_TWO_STAGES) ? TUNE_TWO_STAGES : 0u) |
+         ((flags & COFFEE_FLAG_SUBTILE_64) ? TUNE_SUB64 : 0u) |
+         ((flags & COFFEE_FLAG_SUBTILE_32) ? TUNE_SUB32 : 0u) |
+         ((flags & COFFEE_FLAG_SUBTILE_128) ? TUNE_SUB128 : 0u) |
+         ((flags & COFFEE_FLAG_CELL_LANES) ? TUNE_CELL_LANES : 0u) |
+         ((flags & COFFEE_FLAG_STAGED_STORE) ? TUNE_STAGED_STORE : 0u) |
+         ((flags & COFFEE_FLAG_BURGERS_BLOCKS) ? TUNE_BURGERS_BLOCKS : 0u) |
+         ((flags & COFFEE_FLAG_BURGERS_FACTORED) ? TUNE_BURGERS_FACTORED : 0u) |
+         ((flags & COFFEE_FLAG_KNOB_HINT) ? TUNE_HINT : 0u);
+}
+
 // Local assembly (map == NULL: element matrices to a->out) or fused global assembly
 // (map != NULL: entries added into the CSR values a->out at map[cell][entry]).
 int assemble_impl(const coffee_assemble_args* a, const uint32_t* map, int64_t nnz, coffee_stream_t stream) {
@@ -503,15 +516,7 @@ int assemble_impl(const coffee_assemble_args* a, const uint32_t* map, int64_t nn
   p.aux_off = meta.aux_off;
   p.aux_vparts = meta.aux_vparts;
   p.aux_cparts = meta.aux_cparts;
-  p.tune = ((a->flags & COFFEE_FLAG_OUTPUT_LANES) ? TUNE_OUTPUT_LANES : 0u) |
-           ((a->flags & COFFEE_FLAG_TWO_STAGES) ? TUNE_TWO_STAGES : 0u) |
-           ((a->flags & COFFEE_FLAG_SUBTILE_64) ? TUNE_SUB64 : 0u) |
-           ((a->flags & COFFEE_FLAG_SUBTILE_32) ? TUNE_SUB32 : 0u) |
-           ((a->flags & COFFEE_FLAG_SUBTILE_128) ? TUNE_SUB128 : 0u) |
-           ((a->flags & COFFEE_FLAG_CELL_LANES) ? TUNE_CELL_LANES : 0u) |
-           ((a->flags & COFFEE_FLAG_STAGED_STORE) ? TUNE_STAGED_STORE : 0u) |
-           ((a->flags & COFFEE_FLAG_BURGERS_BLOCKS) ? TUNE_BURGERS_BLOCKS : 0u) |
-           ((a->flags & COFFEE_FLAG_BURGERS_FACTORED) ? TUNE_BURGERS_FACTORED : 0u);
+  p.tune = tune_bits(a->flags);
   p.precision = a->precision;
   p.validate = validate ? 1 : 0;
   p.nu = a->nu;
@@ -875,6 +880,14 @@ int coffee_table_image(int form, int degree, int cell, int precision, uint8_t* i
   }
   if (img) std::memcpy(img, h.data(), h.size());
   return COFFEE_OK;
+}
+
+int coffee_diag_sector_stores(int form, int degree, int cell, int precision, unsigned flags, int64_t out_stride,
+                              int64_t ncells) {
+  if (!valid_fdc(form, degree, cell) || precision < PREC_FP64 || precision > PREC_BF16X3 || out_stride < 0 || ncells < 0)
+    return fail(COFFEE_ERR_INVALID_ARG, "form/degree/cell/precision, out_stride or ncells out of range");
+  const int64_t ns = nnodes(cell, degree);
+  return tc_shift_use(form, degree, cell, precision, out_stride ? out_stride : ns * ns, tune_bits(flags), ncells);
 }
 
 int coffee_diag_wait_timeout(coffee_stream_t stream) {

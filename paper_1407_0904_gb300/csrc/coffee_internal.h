@@ -32,7 +32,9 @@ enum : unsigned { ERR_INDEX = 1u, ERR_TIMEOUT = 2u, ERR_CAPACITY = 4u };
 // Tuning knobs of the tensor-core kernels (from coffee_assemble_args.flags)
 enum : unsigned { TUNE_OUTPUT_LANES = 1u, TUNE_TWO_STAGES = 2u, TUNE_SUB64 = 4u, TUNE_SUB32 = 8u, TUNE_SUB128 = 16u,
                   TUNE_CELL_LANES = 32u, TUNE_STAGED_STORE = 128u, TUNE_BURGERS_BLOCKS = 256u,
-                  TUNE_BURGERS_FACTORED = 512u };
+                  TUNE_BURGERS_FACTORED = 512u, TUNE_HINT = 1024u };
+// the knobs of the kernel with direct or staged stores (k_tc.cu, k_tc_staged.cu)
+constexpr unsigned TUNE_KNOBS = TUNE_OUTPUT_LANES | TUNE_TWO_STAGES | TUNE_SUB64 | TUNE_SUB32 | TUNE_SUB128 | TUNE_CELL_LANES | TUNE_STAGED_STORE;
 
 // ---- host tabulation (tabulate.cpp) ----
 int nnodes(int cell, int k);

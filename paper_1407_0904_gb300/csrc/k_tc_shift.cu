@@ -261,7 +261,8 @@ int tc_shift_possible(int form, int degree, int cell, int precision) {
 }
 
 int tc_shift_use(int form, int degree, int cell, int precision, int64_t ostride, unsigned tune, int64_t ncells) {
-  if (!tc_shift_possible(form, degree, cell, precision) || ostride % 8 == 0 || (tune & TUNE_STAGED_STORE)) return 0;
+  if (!tc_shift_possible(form, degree, cell, precision) || ostride % 8 == 0) return 0;
+  if ((tune & TUNE_KNOBS) && !(tune & TUNE_HINT)) return 0;  // a knob of the other kernel's asks for that kernel
   const ShiftShape s = shift_shape(form, degree, cell, precision);
   return ncells >= (s.mtiles > 4 ? (s.mm > 3 ? 32768 : 16384) : s.mm == 3 ? 131072 : 16384);
 }

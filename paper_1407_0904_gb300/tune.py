@@ -145,7 +145,10 @@ def tune_all(forms=None, cells=(0, 1), degrees=(1, 2, 3, 4), precisions=None, nc
                     simt = coffee.assemble_path(form, k, cell, prec, coffee.FLAG_CUDA_CORES) == 2
                     for t in candidates(coffee, n, simt):
                         times[t] = time_case(coffee, form, k, cell, prec, meshes[cell], t, reps=reps)
-                    best = min(times, key=times.get)
+                    # (0 runs the sector-aligned stores here, which have no knobs: the best knobs are for the launches
+                    # that do not take them, as FLAG_KNOB_HINT says where they are used)
+                    sectors = coffee.diag_sector_stores(form, k, cell, prec, 0, 0, meshes[cell].ncells)
+                    best = min((t for t in times if t or not sectors), key=times.get)
                     key = "%d/%d/%d/%d" % (form, k, cell, prec)
                     entries[key] = {"flags": int(best), "ms": times[best], "ncells": meshes[cell].ncells,
                                     "candidates": {str(t): round(v, 5) for t, v in times.items()}}
