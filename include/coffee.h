@@ -149,7 +149,9 @@ typedef enum {
  * on both cells and for triangles P2, the Burgers forms included; global CSR assembly stays on
  * the tensor cores, batches put the CUDA-core groups in a launch of their own); these flags
  * force one: TENSOR_CORES the tcgen05 kernel, CUDA_CORES the FP32 kernel (ignored where it has
- * no instance). Results of the two differ by rounding, within the precision's bound. */
+ * no instance). Results of the two differ by rounding, within the precision's bound.
+ * In FP64 CUDA_CORES keeps coffee_assemble_ex, coffee_assemble_csr and coffee_assemble_backward
+ * on the plain one-thread-per-cell kernels (see coffee_precision). */
 #define COFFEE_FLAG_TENSOR_CORES 512u
 #define COFFEE_FLAG_CUDA_CORES 1024u
 /* BURGERS_JAC on the tensor cores with component blocks of at most 128 entries (triangles

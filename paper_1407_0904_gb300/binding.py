@@ -484,14 +484,15 @@ def host_pool_trim():
 
 def assemble_backward(form, degree, cell, coords, cell2vert, dout, coef=None, cell2dof=None,
                       precision=FP64, d_coords=None, d_coef=None, deterministic=False,
-                      validate=False, nu=0.01, stream=None):
+                      validate=False, nu=0.01, stream=None, tune=0):
     """Adjoint of assemble: accumulates dL/dcoords (and dL/dcoef) for dout = dL/dA.
 
     dout is float64 for precision FP64 and float32 otherwise. Returns (d_coords, d_coef);
-    tensors passed in are accumulated into (+=), missing ones start at zero."""
+    tensors passed in are accumulated into (+=), missing ones start at zero. tune: FLAG_CUDA_CORES
+    keeps FP64 on the plain kernel."""
     odt = torch.float64 if precision == FP64 else torch.float32
     a, _ = make_args(form, degree, cell, coords, cell2vert, coef, cell2dof, precision,
-                     _dev(dout, odt, "dout"), nu, validate)
+                     _dev(dout, odt, "dout"), nu, validate, tune=tune)
     if d_coords is None:
         d_coords = torch.zeros_like(coords)
     _dev(d_coords, torch.float64, "d_coords")
@@ -510,24 +511,24 @@ class AssembleFn(torch.autograd.Function):
     """Element matrices as a differentiable function of vertex coordinates and coefficients.
 
     AssembleFn.apply(coords, coef, cell2vert, cell2dof, form, degree, cell, precision,
-    deterministic) -> [ncells, ndof, ndof]; backward gives dL/dcoords and dL/dcoef through
-    the library's adjoint kernel (geometry recomputed, not stored)."""
+    deterministic, tune) -> [ncells, ndof, ndof]; backward gives dL/dcoords and dL/dcoef through
+    the library's adjoint kernel (geometry recomputed, not stored). tune as in assemble, for both directions."""
 
     @staticmethod
     def forward(ctx, coords, coef, cell2vert, cell2dof, form, degree, cell, precision=FP64,
-                deterministic=False):
-        out = assemble(form, degree, cell, coords, cell2vert, coef, cell2dof, precision=precision)
+                deterministic=False, tune=None):
+        out = assemble(form, degree, cell, coords, cell2vert, coef, cell2dof, precision=precision, tune=tune)
         ctx.save_for_backward(coords, coef, cell2vert, cell2dof)
-        ctx.meta = (form, degree, cell, precision, deterministic)
+        ctx.meta = (form, degree, cell, precision, deterministic, tune)
         return out
 
     @staticmethod
     def backward(ctx, dout):
         coords, coef, c2v, c2d = ctx.saved_tensors
-        form, degree, cell, precision, deterministic = ctx.meta
+        form, degree, cell, precision, deterministic, tune = ctx.meta
         dc, dk = assemble_backward(form, degree, cell, coords, c2v, dout.contiguous(), coef, c2d,
-                                   precision=precision, deterministic=deterministic)
-        return dc, dk, None, None, None, None, None, None, None
+                                   precision=precision, deterministic=deterministic, tune=tune or 0)
+        return dc, dk, None, None, None, None, None, None, None, None
 
 
 def assemble_backward_noalloc(form, degree, cell, coords, cell2vert, dout, coef=None, cell2dof=None,
