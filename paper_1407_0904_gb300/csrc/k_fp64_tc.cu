@@ -346,9 +346,9 @@ __global__ void __launch_bounds__(F_THREADS, 1) k_assemble_fp64_tc(const Fp64Par
       if (!flag && !scale_of<FORM, D>(G, p.tk20, X, big)) flag = 2;
       if constexpr (FORM != FORM_MASS)
         if (flag == 2) factors64<FORM, D, false>(p, e, G);  // infinities and NaN as divisions give them
-      // Parities tell only neighbouring phases apart. The warps are at most 2 tiles apart and there are 2
-      // stages or more, so the stage's use before this one is the oldest whose tile may still be missing:
-      // once it is full, its release is the phase that the second wait can mean.
+      // Parities tell only neighbouring phases apart. This warp's tile before, i - 3, was stored after tile i - 3 - nst had
+      // been contracted, so with 3 stages or more (one per producer warp) the stage's use before the last, tile i - 2 nst,
+      // is over: the first wait can only mean the last use, tile i - nst, and once that is full, the second its release.
       const uint32_t use = (uint32_t)(i / nst);
       const uint32_t n = (uint32_t)(i / F_PROD);  // of this warp's tiles
       bool ok = use == 0 || mbar_wait(full + 8 * st, (use - 1) & 1u, p.err);
@@ -575,7 +575,9 @@ constexpr int F_FIXED = F_HALVES * F_XRING * FN * 8 + F_HALVES * F_PROD * 64 * 4
 template <int FORM, int D>
 int fit_slices(int mtiles) {
   using DG = Digits<FORM, D>;
-  const int fit = (F_SMEM_LIMIT - F_FIXED - F_HALVES * 2 * DG::STAGE) / DG::SLICE;
+  // a stage for every producer warp (see the waits there)
+  static_assert(F_SMEM_LIMIT - F_FIXED - F_HALVES * F_PROD * DG::STAGE >= DG::SLICE && F_STAGES >= F_PROD, "stages");
+  const int fit = (F_SMEM_LIMIT - F_FIXED - F_HALVES * F_PROD * DG::STAGE) / DG::SLICE;
   if (fit >= mtiles) return mtiles;
   const int groups = (mtiles + fit - 1) / fit;  // even shares
   return (mtiles + groups - 1) / groups;
