@@ -447,6 +447,11 @@ __global__ void __launch_bounds__(G_THREADS, 1) k_backward_tc(const BwdParams p)
         mbar_arrive(full + 8 * st);
       }
     }
+    // no copy may land after this block has left (its waits may have expired): wait for the last one of each stage
+    if (w == 0 && lane == 0)
+      for (uint32_t k = n > (uint32_t)AF::STAGES ? n - AF::STAGES : 0; k < n; ++k)
+        mbar_wait(full + 8 * (k % AF::STAGES), (k / AF::STAGES) & 1u, p.err);
+    __syncwarp();
   } else if (warp >= G_EPI + G_PROD && warp < G_WARPS - 1) {
     // ---------------- scan: the largest exponent of every cell's dA in a drain's entries, drains ahead ----------------
     // A drain's error is 2^-55 of max|T[k]| times its own largest |dA|: no more than roundings of sum_o |T[k][o] dA[o]| where a
