@@ -243,7 +243,7 @@ def prism_fma(form, k):
     if form == BURGERS_RESIDUAL:
         return point + p ** 3 * nz * 12 + p * p * nt * nz * 9
     ntp, nzp = nt * (nt + 1) // 2, nz * (nz + 1) // 2
-    fields, per = {MASS: (1, 1), HELMHOLTZ: (9, 8), ADVDIFF: (12, 11), BURGERS_JAC: (21, 20)}[form]
+    fields, per = {MASS: (1, 1), HELMHOLTZ: (9, 8), ADVDIFF: (12, 13), BURGERS_JAC: (21, 22)}[form]
     return point + p ** 3 * nzp * fields + p * p * ntp * nzp * per
 
 
@@ -592,9 +592,9 @@ def run_ours(args):
             # tensor pipe: executed MMA flops, one pass per product of operand parts the kernel keeps, against the
             # tf32/bf16 dense peak
             tf32 = prec in (coffee.TF32, coffee.TF32X3)
-            if form in (HELMHOLTZ, ADVDIFF):
+            if form in (HELMHOLTZ, ADVDIFF) and prec == coffee.TF32X3:
                 # summed over z first: 8 columns a triangle point and the centre's (two points a chunk), 128 rows a
-                # tile of a lane quadrant's cells times four, split tf32 whatever the precision
+                # tile of a lane quadrant's cells times four
                 nt, nz, qt = (degree + 1) * (degree + 2) // 2, degree + 1, (degree + 2) ** 2
                 rows = nz * (nz + 1) // 2 if form == HELMHOLTZ else nz * nz
                 flops = 2.0 * 8 * qt * (rows * nt * nt + (degree + 2) * rows) + 250.0 * Q
@@ -618,12 +618,14 @@ def run_ours(args):
                     "executed_flops_per_cell": executed, "algorithmic_flops_per_cell": flops,
                     "kernel_ms": launch_ms, "hbm_gbs": achieved}
 
-    fp64 = None
+    # the same workload in FP64, by the library's own choice of kernel and on the plain one-thread-per-cell kernel
+    fp64 = plain64 = None
     if prec != coffee.FP64 and not args.no_fp64:
         out64 = torch.empty(tuple(out.shape), dtype=torch.float64, device=dev)  # same row layout
         fsteps = max(3, min(args.steps // 20, 100))
-        tms, lms = timed(lambda: step(coffee.FP64, out64, coffee.FLAG_CUDA_CORES), fsteps, 3)
-        fp64 = {"value": ncells * fsteps / (tms / 1e3), "kernel_ms": lms, "steps": fsteps}
+        run64 = lambda flags: timed(lambda: step(coffee.FP64, out64, flags), fsteps, 3)
+        fp64, plain64 = ({"value": ncells * fsteps / (tms / 1e3), "kernel_ms": lms, "steps": fsteps}
+                         for tms, lms in (run64(None), run64(coffee.FLAG_CUDA_CORES)))
         del out64
 
     # end to end through the public API with host buffers
@@ -700,7 +702,7 @@ def run_ours(args):
                            "coordinates": ("split into float (hi, lo) pairs once per vertex each step "
                                            "(coffee_split_coords, timed with the assembly)" if xsplit is not None
                                            else "FP64, split per cell in the kernel")},
-                "roofline": roof, "fp64_kernel": fp64,
+                "roofline": roof, "fp64_kernel": fp64, "fp64_plain_kernel": plain64,
                 "tc_vs_fp64": (value / world / fp64["value"]) if fp64 else None,
                 "e2e": e2e, "cpu_baseline": cpu, "gpu_launches": args.steps * launches_per_step,
                 "clocks": clocks, "kernel_sha": sha, "device_peaks": device_peaks(coffee),
