@@ -216,7 +216,9 @@ def _address(t):
 
 def _stream_handle(stream):
     if stream is None:  # the current device's current stream, without a Stream object made for each call
-        return ctypes.c_void_p(torch._C._cuda_getCurrentRawStream(torch.cuda.current_device()))
+        dev = torch.cuda.current_device()
+        raw = getattr(torch._C, "_cuda_getCurrentRawStream", None)  # (not a public name)
+        return ctypes.c_void_p(raw(dev) if raw is not None else torch.cuda.current_stream(dev).cuda_stream)
     return ctypes.c_void_p(stream.cuda_stream)
 
 
