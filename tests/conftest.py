@@ -20,6 +20,9 @@ def pytest_sessionstart(session):
 
 
 def pytest_collection_modifyitems(config, items):
+    # test_around_a_tile wants prisms in TF32, BF16 and BF16X3 bit-equal to TF32X3, which include/coffee.h's definition of
+    # those precisions rules out: its last two lines fail. Run at the end, so that -x has run everything else by then.
+    items.sort(key=lambda it: it.name.startswith("test_around_a_tile["))
     try:
         import torch
         has_gpu = torch.cuda.is_available()
