@@ -41,13 +41,13 @@
 // into groups by 128-entry slices, each with its slices resident, and form the factors once per group.
 // What bounds it now is the integer work of the epilogue, about 26 instructions an entry (half of them
 // moved to the multiplier pipe, see mad_lo), and the latencies between its phases; for advection-diffusion the
-// producers. 196,608 perturbed tetrahedra (thin layers), this kernel / plain: Helmholtz P2 80 (184) / 302 us, P3 155
-// (427) / 1140 us, 0.6 of the copy bandwidth, P4 384 (1106) / 3480 us; advection-diffusion P1 184 (290) / 276, P2 204
-// (615) / 1450 us, P3 0.81 (2.59) / 5.41 ms. Steps on the way (Helmholtz P3): one
+// producers. 196,608 perturbed tetrahedra (thin layers), this kernel / plain: Helmholtz P2 80 (193) / 302 us, P3 155
+// (477) / 1140 us, 0.6 of the copy bandwidth, P4 381 (1230) / 3480 us; advection-diffusion P1 175 (280) / 276, P2 183
+// (559) / 1450 us, P3 0.76 (2.31) / 5.41 ms. Steps on the way (Helmholtz P3): one
 // pipeline with 21 warps 479 us; 16 warps of 128 registers 324; multiplications for shifts 311; two
 // pipelines 242; 16 cells per epilogue warp, four epilogue warps a scheduler, 169; one wide MMA per digit of T
 // instead of one per order and K step 158 (advection-diffusion P2 168 -> 123). The masks and weak_entries took
-// advection-diffusion P2 from 123 to 204 us and Helmholtz P2 from 59 to 80.
+// advection-diffusion P2 from 123 to 183 us and Helmholtz P2 from 59 to 80.
 #include <cuda_runtime.h>
 #include <cuda_fp16.h>
 #include <algorithm>
@@ -116,7 +116,7 @@ __device__ constexpr bool leaves() { return CSR || (FORM == FORM_ADVDIFF && D ==
 // in classes of one mask of large table entries, whose rows of T lie one after the other, the entry's number last.
 // Few cells fail a class (perturbed tetrahedra: 40 pairs of a cell and an entry in a tile), so pairs are queued and summed
 // 32 at a time, a pair per lane with the factors from their cell's lane: class by class for all lanes, advection-diffusion
-// P2 on 196,608 tetrahedra took 415 us, now 204. Called by whole warps, and every lane takes part in every
+// P2 on 196,608 tetrahedra took 415 us, now 183. Called by whole warps, and every lane takes part in every
 // exchange; false on expiry.
 template <int FORM, int D, bool CSR>
 __device__ __forceinline__ bool weak_entries(const Fp64Params& p, int64_t e0, bool live, uint32_t big,
@@ -176,35 +176,44 @@ __device__ __forceinline__ bool weak_entries(const Fp64Params& p, int64_t e0, bo
     }
     __syncwarp();
   };
-  for (int c0 = range.x; c0 < range.y; c0 += 32) {
-    // 32 classes on the lanes (mask, first row, last row + 1): those that not every cell has a large factor of
-    const int4 cl = c0 + lane < range.y ? __ldg(classes + c0 + lane) : make_int4(-1, 0, 0, 0);
-    for (uint32_t hits = __ballot_sync(FULL, (common & (uint32_t)cl.x) == 0u && cl.y < cl.z); hits; hits &= hits - 1) {
-      const int src = __ffs(hits) - 1;
-      const uint32_t mask = (uint32_t)__shfl_sync(FULL, cl.x, src);
-      const int first = __shfl_sync(FULL, cl.y, src), last = __shfl_sync(FULL, cl.z, src);
-      const uint32_t fails = __ballot_sync(FULL, live && (big & mask) == 0u);
-      if (fails == 0u) continue;
-      if (!waited) {
-        if (!__all_sync(FULL, mbar_wait(stored, n & 1u, p.err))) return false;
-        waited = true;
-      }
-      const int count = __popc(fails);
-      for (int i = first; i < last; ++i) {
-        if (fails >> lane & 1u) queue[queued + __popc(fails & ((1u << lane) - 1u))] = (uint32_t)i << 5 | (uint32_t)lane;
-        queued += count;
-        if (queued >= 32) {
-          flush(32);
-          queued -= 32;
-          const uint32_t rest = queue[32 + lane];
-          __syncwarp();
-          if (lane < queued) queue[lane] = rest;
+  // (one place that sums: inlined twice, advection-diffusion's code waited for instructions, P2 205 us)
+  int4 cl = make_int4(0, 0, 0, 0);   // 32 classes on the lanes: mask, first row, last row + 1
+  uint32_t hits = 0, fails = 0;      // of them, those that not every cell has a large factor of; the cells that fail the class
+  int c0 = range.x, i = 0, last = 0;  // next classes, next row of the class
+  for (;;) {
+    while (queued < 32) {
+      if (i == last) {
+        for (; hits == 0u && c0 < range.y; c0 += 32) {
+          cl = c0 + lane < range.y ? __ldg(classes + c0 + lane) : make_int4(-1, 0, 0, 0);
+          hits = __ballot_sync(FULL, (common & (uint32_t)cl.x) == 0u && cl.y < cl.z);
         }
+        if (hits == 0u) break;
+        const int src = __ffs(hits) - 1;
+        hits &= hits - 1;
+        const uint32_t mask = (uint32_t)__shfl_sync(FULL, cl.x, src);
+        i = __shfl_sync(FULL, cl.y, src);
+        last = __shfl_sync(FULL, cl.z, src);
+        fails = __ballot_sync(FULL, live && (big & mask) == 0u);
+        if (fails == 0u) i = last;
+        continue;
       }
+      if (fails >> lane & 1u) queue[queued + __popc(fails & ((1u << lane) - 1u))] = (uint32_t)i << 5 | (uint32_t)lane;
+      queued += __popc(fails);
+      ++i;
     }
+    if (queued == 0) return true;
+    if (!waited) {
+      if (!__all_sync(FULL, mbar_wait(stored, n & 1u, p.err))) return false;
+      waited = true;
+    }
+    const int count = queued < 32 ? queued : 32;
+    flush(count);
+    queued -= count;
+    const uint32_t rest = queue[32 + lane];
+    __syncwarp();
+    if (lane < queued) queue[lane] = rest;
+    __syncwarp();
   }
-  if (queued) flush(queued);
-  return true;
 }
 
 // The largest biased exponent X of a cell's scaled factors, in place (<< 20; 0: all are zero), and the mask `big` of those
@@ -677,8 +686,8 @@ void image_of(int degree, int cell, std::vector<uint8_t>& img, Fp64Image& h) {
 
 // Where the digit contraction runs instead of the plain kernel: where it is the faster one at every count of cells
 // from 300 (both launch-bound, 8-20 us against 11-2300 us) and on perturbed meshes as on thin layers, or nearly so. us,
-// 196,608 cells perturbed, layered / plain: advection-diffusion P1 tetrahedra 184, 290 / 276, P2 triangles 70, 122 / 223;
-// Helmholtz P2 tetrahedra 80, 184 / 302, P4 triangles 87, 156 / 570. Left to the plain kernel are
+// 196,608 cells perturbed, layered / plain: advection-diffusion P1 tetrahedra 175, 280 / 276, P2 triangles 70, 123 / 223;
+// Helmholtz P2 tetrahedra 80, 193 / 302, P4 triangles 87, 182 / 570. Left to the plain kernel are
 // Helmholtz on fewer than 10 nodes (P2 triangles 70, 119 / 76, P1 tetrahedra 74, 107 / 86, P1 triangles 47 / 32) and the
 // mass matrices of up to 6 nodes (one multiplication an entry: P2 triangles at 300 cells 5 against 9 us).
 int fp64_tc_use(int form, int degree, int cell) {
