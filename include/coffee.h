@@ -70,7 +70,9 @@ typedef struct CUstream_st* coffee_stream_t;
  * and ADVDIFF (eps and b given per vertex through cell2dof [ncells][6], evaluated at each point
  * with the degree-1 prism functions): FP64 and the tensor-core precisions for P1-P4
  * (the contraction over all quadrature points is streamed through shared memory in K-chunks,
- * at most three 128-output slices at a time),
+ * at most three 128-output slices at a time; TF32X3 element matrices of HELMHOLTZ and ADVDIFF are
+ * summed over z first, then over the triangle's points, so that they differ by rounding, within the
+ * precision's bound, from what coffee_assemble_csr adds up),
  * both through coffee_assemble_ex and coffee_assemble_csr. The Burgers Jacobian and residual on
  * prisms (u per node through cell2dof [ncells][(k+1)^2(k+2)/2], rows and columns blocked by
  * component as on simplices) run in FP64 with their own rule of (3k+3)/2 points per direction

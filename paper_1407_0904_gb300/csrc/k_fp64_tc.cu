@@ -1,5 +1,6 @@
 // FP64 local and global assembly on the tensor cores: A_e[o] = sum_k G_e[k] T[k][o] with the
-// contraction done exactly, in integers, by tcgen05 f16 MMAs.
+// contraction done exactly, in integers, by tcgen05 f16 MMAs. (Matrix products from slices whose products are exact:
+// Ozaki, Ogita, Oishi and Rump, Numerical Algorithms 59 (2012), 95-118.)
 //
 // What bounds the plain FP64 kernel is the FP64 pipe, 2 FMAs per cycle and SM on this GPU: Helmholtz
 // P3 on tetrahedra (K = 7 FMAs for each of 400 entries) takes 1400 cycles a cell, ten times the 150

@@ -16,8 +16,9 @@
 // Only TF32X3: the other precisions are defined by the parts that each point's factors are held in, and sums over z
 // rounded to those parts are other numbers (TF32 here and there: 3e-4 of the entries apart).
 // Bound by shared memory (L1 data pipe 72 % busy beside the MMAs' operands, 78 of 7.5 KB a P3 tile) and, with it, the
-// latency of the fields' and the epilogue's chains: a seventh fewer wavefronts by padding gained 2 % at P3, lost 3 % at P1. Factors and fields are separate warps, two tiles of factors in flight,
-// because in the same warps one after the other they took 24,000 cycles a P3 tile for 16,800; matrix rows put
+// latency of the fields' and the epilogue's chains: a seventh fewer wavefronts by padding gained 2 % at P3, lost 3 % at P1.
+// Factors and fields are separate warps, two tiles of factors in flight, because in the same warps one after the other
+// they took 24,000 cycles a P3 tile (15,400 now); matrix rows put
 // together in shared memory because stores of a thread's own runs of nt entries touch 32 sectors each (P4: 48,000
 // cycles a tile of stores, 22,000 now).
 //
