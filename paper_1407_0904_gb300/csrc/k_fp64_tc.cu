@@ -28,9 +28,11 @@
 // leaves that entry out (weak_entries). Elsewhere sum_k |G_k T_k| is at least 2^-8 of the product of the largest. The
 // cost goes with what it does: 0.4 % of the entries of perturbed P3 tetrahedra, a fifth to a half of them on thin
 // layers, all entries of cells whose factors are not finite or outside 2^+-900, which have no digits.
-// Error of an entry relative to its own sum_k |G_k T_k|, largest and rms in units of 2^-53, this kernel / plain:
-// perturbed tetrahedra Helmholtz P3 1.4, 0.23 / 2.5, 0.36, advection-diffusion P2 4.7, 0.58 / 5.0, 0.64; layers of 1/1000
-// 2.5, 0.34 / 3.7, 0.51 and 6.1, 0.62 / 6.6, 0.87 (without the masks 5e7 and 1e8).
+// Error of an entry against quadruple precision relative to its own sum_k |G_k T_k|, rms in units of 2^-53, this kernel /
+// plain: Helmholtz P3 tetrahedra perturbed 0.90 / 0.94, right-angled 0.24 / 0.34; advection-diffusion P2 perturbed 1.32 /
+// 1.38, right-angled 0.43 / 0.62, with eps = 1e-6 0.56 / 0.59; P3 triangles 0.51 / 0.71, in layers of 1/1000 0.72 / 0.88. No
+// rms is larger; the largest errors are the same (the factors' own) or within 1.2 times, but for triangles in layers,
+// 11 / 5.6. Without the masks the largest were 1e4 (right-angled) to 1e8 (layers).
 //
 // Operands are K-major without swizzle: 16-byte rows (8 factors of one digit) contiguous in chunks; T by
 // 128-entry slice, digit and chunk, the cells by chunk, digit and cell (see the MMA warp for why).
