@@ -18,8 +18,8 @@
 // plain kernel's or smaller (1.0e-15 and 1.1e-15 for advection-diffusion P2).
 // An error relative to the largest dA of a row is a rounding of Gbar[k]'s own terms only if some large dA meets a large
 // T[k]. The scan looks for one for every k; cells without (one entry far above the others, a single row of dA) take
-// the plain sums, alone by the scan's warp (whole_cell), many by a lane each (plain_gbar, 1.1-1.2 times the plain
-// kernel's time when all are). The check costs up to a quarter: us for 196,608 tetrahedra without / with it, advection-
+// the plain sums, alone by the scan's warp (whole_cell), many by a lane each (plain_gbar: with one row of dA alone
+// in every cell 0.3-1.1 times the plain kernel's time on tetrahedra, with six decades of spread 1.2-1.5). The check costs up to a quarter: us for 196,608 tetrahedra without / with it, advection-
 // diffusion P1 164 / 221, P2 193 / 206, P3 584 / 670, Helmholtz P1 88 / 104, P2 124 / 128.
 //   warps 0-7    epilogue, two sets on alternate tiles (one drains while the other is in the FP64 chain);
 //                a thread has one cell: drains, chain rule, atomics or local rows
@@ -139,13 +139,25 @@ __device__ __noinline__ void plain_gbar(const BwdParams& p, int64_t e, double* G
   double s[KP];
 #pragma unroll
   for (int k = 0; k < KP; ++k) s[k] = 0.0;
-  for (int o = 0; o < p.N; ++o) {
-    const double a = __ldg(row + o);
+  constexpr int U = K <= 16 ? 4 : 1;  // entries whose loads are issued together
+  for (int o = 0; o < p.N; o += U) {
+    double a[U];
+    bool some = false;
 #pragma unroll
-    for (int k = 0; k < KP; k += 2) {
-      const double2 t = __ldg(T + o * (KP / 2) + k / 2);
-      s[k] = fma(t.x, a, s[k]);
-      s[k + 1] = fma(t.y, a, s[k + 1]);
+    for (int j = 0; j < U; ++j) {
+      a[j] = o + j < p.N ? __ldg(row + o + j) : 0.0;
+      some = some || a[j] != 0.0;
+    }
+    if (!some) continue;  // (dA of a few rows or columns is what comes here most)
+#pragma unroll
+    for (int j = 0; j < U; ++j) {
+      const int r = U == 1 || o + j < p.N ? o + j : o;  // past the end: any row, by zero
+#pragma unroll
+      for (int k = 0; k < KP; k += 2) {
+        const double2 t = __ldg(T + r * (KP / 2) + k / 2);
+        s[k] = fma(t.x, a[j], s[k]);
+        s[k + 1] = fma(t.y, a[j], s[k + 1]);
+      }
     }
   }
 #pragma unroll
